@@ -10,9 +10,14 @@
 #include <new>
 #include <vector>
 
+#include "sq_quad.cuh"
 #include "sq_queue.cuh"
 
 namespace sq {
+int quad_config(int m, int which, bool has_nl, int ccap, int lb, int npl, size_t* smem);
+int quad_launch(int m, int which, const QuadArgs& a, size_t smem, int blocks, cudaStream_t st);
+int quad_queue_config(int m, int which, size_t smem);
+int quad_queue_launch(int m, int which, const QuadQueueArgs& q, size_t smem, int blocks, cudaStream_t st);
 int region_config_f32(int m, int which, size_t extra, int* bps, size_t* smem);
 int region_config_f64(int m, int which, size_t extra, int* bps, size_t* smem);
 int region_launch_f32(int m, int which, const RegionArgs<float>& a, size_t extra, int blocks, cudaStream_t st);
@@ -82,7 +87,7 @@ int dev_alloc(P** p, size_t bytes)
 void free_ctx(sq_ctx* c)
 {
     if (!c) return;
-    void* ptrs[] = {c->Vp, c->d_atoms, c->d_G, c->d_DG, c->d_ivl, c->d_tile_start, c->d_tile_cand, c->d_scratch,
+    void* ptrs[] = {c->Vp, c->d_atoms, c->d_G, c->d_DG, c->d_ivl, c->d_tile_start, c->d_tile_cand, c->d_scratch, c->d_qscratch, c->d_qmask,
                     c->d_alpha, c->d_beta, c->d_klen, c->d_W, c->d_red, c->d_fermi, c->d_count, c->d_err};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -268,6 +273,57 @@ int cluster_launch(sq_ctx* c, int which, const RegionArgs<float>& a, int blocks)
                        : cluster_launch_f32_hi(c->g.m, which, a, clusters, c->cl_smem[which], c->stream);
 }
 
+// FP32 quad kernels (sq_quad.cuh) for this context: every region half-width
+// that has one, unless its projector tables do not fit next to the vector or
+// SQ_REGION_KERNEL=cta in the environment asks for the general kernels.
+// Allocates their per-CTA scratch and sets c->quad.
+int select_quad_kernels(sq_ctx* c)
+{
+    c->quad = 0;
+    if (c->precision != SQ_FP32 || c->cl_nc > 0) return SQ_OK;
+    const char* env = getenv("SQ_REGION_KERNEL");
+    if (env && strcmp(env, "cta") == 0) return SQ_OK;
+    const bool has_nl = c->n_atoms > 0;
+    if (c->g.m < (has_nl ? QD_MIN_NL : QD_MIN_LOCAL)) return SQ_OK;
+    for (int which = 0; which < 2; ++which) {
+        const int rc = quad_config(c->g.m, which, has_nl, c->ccap, c->lb, c->npl, &c->q_smem[which]);
+        if (rc == SQ_EUNSUPPORTED) return SQ_OK;
+        if (rc) return rc;
+    }
+    c->q_stride = quad_scratch(c->g.m, has_nl ? c->ccap : 0, has_nl ? c->lb : 0).total;
+    int rc = dev_alloc(&c->d_qscratch, c->q_stride * (size_t)c->sm_count);       // one CTA per SM, a queue's too
+    if (rc) return rc;
+    if (has_nl) {
+        if ((rc = dev_alloc(&c->d_qmask, sizeof(uint32_t) * c->lb * c->lb * (size_t)c->n_atoms))) return rc;
+        if ((rc = launch_support_masks(c))) return rc;
+    }
+    c->quad = 1;
+    return SQ_OK;
+}
+
+// Arguments of the quad kernels with the region arguments a.
+QuadArgs quad_args(const sq_ctx* c, const RegionArgs<float>& a)
+{
+    QuadArgs q;
+    memset(&q, 0, sizeof(q));
+    q.r = a;
+    for (int d = 0; d <= FD_NO; ++d) q.wd2[d] = make_float2(a.wd[d], a.wd[d]);
+    q.diag = (float)(-3.0 * c->g.w[0]);
+    q.scratch = (char*)c->d_qscratch;
+    q.stride = c->q_stride;
+    q.mask = c->d_qmask;
+    q.nxq = quad_nxq(c->lb);
+    q.nyp = quad_nyp(c->lb);
+    q.recs = quad_recs(c->lb);
+    return q;
+}
+
+// Launch quad kernel `which` with the region arguments a.
+int launch_quad(sq_ctx* c, int which, const RegionArgs<float>& a, int blocks)
+{
+    return quad_launch(c->g.m, which, quad_args(c, a), c->q_smem[which], blocks, c->stream);
+}
+
 // Dynamic shared memory beyond the region vectors: the moments kernel (which
 // = 0) keeps its per-node moment sums there; both keep the projector tables
 // there when they fit.
@@ -282,6 +338,10 @@ int region_blocks(sq_ctx* c, int which, int* blocks)
         long long b = (long long)c->cl_clusters[which] * c->cl_nc;
         if (b > c->g.Nd * c->cl_nc) b = c->g.Nd * c->cl_nc;
         *blocks = (int)b;
+        return SQ_OK;
+    }
+    if (c->quad) {
+        *blocks = (int)std::min<long long>(c->sm_count, c->g.Nd);
         return SQ_OK;
     }
     int bps = 0;
@@ -323,6 +383,7 @@ int enqueue_bounds(sq_ctx* c, int blocks, int n_lanczos, double margin, double* 
         RegionArgs<float> a = region_args<float>(c);
         a.n_lanczos = n_lanczos; a.nl_cap = c->nl_cap; a.alpha = c->d_alpha; a.beta = c->d_beta; a.klen = c->d_klen;
         rc = c->cl_nc > 0 ? cluster_launch(c, 1, a, blocks)
+             : c->quad    ? launch_quad(c, 1, a, blocks)
                           : region_launch_f32(c->g.m, 1, a, region_extra(c, 1), blocks, c->stream);
     } else {
         RegionArgs<double> a = region_args<double>(c);
@@ -342,6 +403,7 @@ int enqueue_moments(sq_ctx* c, int blocks, const double* chi, const double* zeta
         RegionArgs<float> a = region_args<float>(c);
         a.chi = chi; a.zeta = zeta; a.moments = moments;
         rc = c->cl_nc > 0 ? cluster_launch(c, 0, a, blocks)
+             : c->quad    ? launch_quad(c, 0, a, blocks)
                           : region_launch_f32(c->g.m, 0, a, region_extra(c, 0), blocks, c->stream);
     } else {
         RegionArgs<double> a = region_args<double>(c);
@@ -382,7 +444,7 @@ struct sq_batch {
     int wait_unset = 0;
     // queue plan: groups of systems with one region half-width and precision
     struct Group {
-        int m = 0, prec = SQ_FP32;
+        int m = 0, prec = SQ_FP32, quad = 0;     // quad: its contexts run the quad kernels
         std::vector<int> sys;                    // batch indices, at most QMAX
         int bl = 0, bm = 0;                      // grids of the Lanczos and moments queue kernels
         size_t xl = 0, xm = 0;                   // their dynamic shared memory beyond the region vectors
@@ -537,31 +599,42 @@ int batch_build_queue(sq_batch* b, int npi)
         const sq_ctx* c = b->ctx[i];
         sq_batch::Group* g = nullptr;
         for (auto& x : G)
-            if (x.m == c->g.m && x.prec == c->precision && (int)x.sys.size() < QMAX) g = &x;
+            if (x.m == c->g.m && x.prec == c->precision && x.quad == c->quad && (int)x.sys.size() < QMAX) g = &x;
         if (!g) {
             G.emplace_back();
             g = &G.back();
             g->m = c->g.m;
             g->prec = c->precision;
+            g->quad = c->quad;
         }
         g->sys.push_back(i);
     }
     std::vector<QItem> items;
     for (auto& g : G) {
         for (int i : g.sys) {
+            if (g.quad) {                        // xl, xm: all of the dynamic shared memory
+                g.xl = std::max(g.xl, b->ctx[i]->q_smem[1]);
+                g.xm = std::max(g.xm, b->ctx[i]->q_smem[0]);
+                continue;
+            }
             g.xl = std::max(g.xl, region_extra(b->ctx[i], 1));
             g.xm = std::max(g.xm, region_extra(b->ctx[i], 0));
         }
         int bpl = 0, bpm = 0;
         size_t sm = 0;
         int rc;
-        if ((rc = queue_config(g.prec, g.m, 1, g.xl, &bpl, &sm)) || (rc = queue_config(g.prec, g.m, 0, g.xm, &bpm, &sm)))
+        if (g.quad) {
+            if ((rc = quad_queue_config(g.m, 1, g.xl)) || (rc = quad_queue_config(g.m, 0, g.xm))) return rc;
+            bpl = bpm = 1;
+        } else if ((rc = queue_config(g.prec, g.m, 1, g.xl, &bpl, &sm)) ||
+                   (rc = queue_config(g.prec, g.m, 0, g.xm, &bpm, &sm))) {
             return rc;
+        }
         const int sms = b->ctx[g.sys[0]]->sm_count;
         g.bl = bpl * sms;
         g.bm = bpm * sms;
         for (int i : g.sys)
-            if ((rc = ensure_scratch(b->ctx[i], std::max(g.bl, g.bm)))) return rc;
+            if (!g.quad && (rc = ensure_scratch(b->ctx[i], std::max(g.bl, g.bm)))) return rc;
         const int ns = (int)g.sys.size();
         g.need.assign(ns, 0);
         g.off_l = (int)items.size();
@@ -618,6 +691,31 @@ int queue_launch(int m, int which, const QueueArgs<double>& q, size_t extra, int
     return queue_launch_f64(m, which, q, extra, blocks, st);
 }
 
+// One launch of a queue over the systems of a group (quad kernels where its contexts run them).
+template <typename T>
+int queue_launch(const sq_batch* b, const sq_batch::Group& g, int which, const QueueArgs<T>& q)
+{
+    return queue_launch(g.m, which, q, which ? g.xl : g.xm, which ? g.bl : g.bm, b->own);
+}
+int queue_launch(const sq_batch* b, const sq_batch::Group& g, int which, const QueueArgs<float>& q)
+{
+    if (!g.quad) return queue_launch(g.m, which, q, which ? g.xl : g.xm, which ? g.bl : g.bm, b->own);
+    QuadQueueArgs d;
+    memset(&d, 0, sizeof(d));
+    for (int k = 0; k < (int)g.sys.size(); ++k) {
+        d.sys[k] = quad_args(b->ctx[g.sys[k]], q.sys[k]);
+        d.V[k] = q.V[k];
+        d.need[k] = q.need[k];
+    }
+    d.items = q.items;
+    d.n_items = q.n_items;
+    d.next = q.next;
+    d.done = q.done;
+    d.budget = q.budget;
+    d.unset = q.unset;
+    return quad_queue_launch(g.m, which, d, which ? g.xl : g.xm, which ? g.bl : g.bm, b->own);
+}
+
 // Enqueue group gi of the queue plan on b->own: the Lanczos queue (QI_VPAD
 // items, then the nodes), the tridiagonal extremes of its systems, the
 // moments queue; then fork each system's Fermi search and density onto its
@@ -644,7 +742,7 @@ int batch_enqueue_group(sq_batch* b, int gi, const BatchArgs& A)
     q.done = ctl + 2;
     q.budget = b->wait_budget;
     q.unset = b->wait_unset;
-    int rc = queue_launch(g.m, 1, q, g.xl, g.bl, b->own);
+    int rc = queue_launch(b, g, 1, q);
     if (rc) return rc;
     for (int k = 0; k < ns; ++k) {
         sq_ctx* c = b->ctx[g.sys[k]];
@@ -662,7 +760,7 @@ int batch_enqueue_group(sq_batch* b, int gi, const BatchArgs& A)
     q.items = b->d_items + g.off_m;
     q.n_items = g.n_m;
     q.next = ctl + 1;
-    rc = queue_launch(g.m, 0, q, g.xm, g.bm, b->own);
+    rc = queue_launch(b, g, 0, q);
     if (rc) return rc;
     if (cudaEventRecord(b->gfork[gi], b->own) != cudaSuccess) return SQ_ECUDA;
     for (int k = 0; k < ns; ++k) {
@@ -931,6 +1029,7 @@ int sq_setup_grid(sq_ctx** out, int n1, int n2, int n3, double h, int fd_half_or
     c->scratch_bytes_per_cta = scratch_layout(m, tsz).total;
     if (c->cl_nc == 0 &&               // the cluster kernels keep everything in shared memory
         (rcode = dev_alloc(&c->d_scratch, c->scratch_bytes_per_cta * c->grid_blocks))) { free_ctx(c); return rcode; }
+    if ((rcode = select_quad_kernels(c))) { free_ctx(c); return rcode; }
     c->red_blocks = c->sm_count * 4;
     if ((rcode = dev_alloc(&c->d_W, sizeof(double) * c->g.Nd * (npl + 1))) ||
         (rcode = dev_alloc(&c->d_red, sizeof(double) * 3 * c->red_blocks)) ||

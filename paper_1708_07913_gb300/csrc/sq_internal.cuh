@@ -157,6 +157,14 @@ struct sq_ctx {
     int cl_nc;
     int cl_clusters[2];
     size_t cl_smem[2];
+    // FP32 quad region kernels (sq_quad.cuh), one CTA per SM: in use (0: the
+    // general single-CTA kernels), their dynamic shared memory per kernel (0
+    // moments, 1 Lanczos) and per-CTA scratch
+    int quad;
+    size_t q_smem[2];
+    void* d_qscratch;
+    uint32_t* d_qmask;               // support rows as column masks (QuadArgs::mask)
+    size_t q_stride;
     // per-CTA scratch
     int grid_blocks;                 // resident CTAs used for the region kernels
     size_t scratch_bytes_per_cta;
@@ -192,6 +200,7 @@ int enqueue_density(sq_ctx* ctx, const double* chi, const double* zeta, double m
 constexpr int FERMI_STATE = 12;      // doubles of the device Fermi/energy state
 int fermi_result(const double* st_host, double* mu, double* eb, double* es, double* ne);
 int launch_proj_tables(sq_ctx* ctx, const double* d_R);
+int launch_support_masks(sq_ctx* ctx);
 }  // namespace sq
 
 #define SQ_CUDA_TRY(call)                                   \

@@ -103,6 +103,28 @@ int launch_proj_tables(sq_ctx* ctx, const double* d_R)
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
 
+// Support rows as 32-bit column masks, [atom][plane kk][row jj] (boxes have at
+// most NL_BOX = 32 columns): what the quad kernels cut their lists from.
+__global__ void support_mask_kernel(const uint8_t* __restrict__ ivl, int n_atoms, int lb, uint32_t* __restrict__ mask)
+{
+    const long long n = (long long)n_atoms * lb * lb;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
+        const int jj = (int)(t % lb), kk = (int)((t / lb) % lb);
+        const long long atom = t / ((long long)lb * lb);
+        const uchar2 iv = *reinterpret_cast<const uchar2*>(ivl + ((atom * lb + jj) * lb + kk) * 2);
+        mask[t] = iv.x <= iv.y ? (0xffffffffu >> (31 - iv.y)) & (0xffffffffu << iv.x) : 0u;
+    }
+}
+
+int launch_support_masks(sq_ctx* ctx)
+{
+    const long long n = (long long)ctx->n_atoms * ctx->lb * ctx->lb;
+    support_mask_kernel<<<(int)std::min<long long>((n + 255) / 256, (long long)ctx->sm_count * 8), 256, 0, ctx->stream>>>(
+        ctx->d_ivl, ctx->n_atoms, ctx->lb, ctx->d_qmask);
+    ctx->launches++;
+    return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
+}
+
 // ------------------------------------------------------------------------
 // Extreme eigenvalues of the Lanczos tridiagonal T_k by Sturm bisection.
 // The count of eigenvalues below x is the number of sign changes of the
