@@ -1032,7 +1032,7 @@ int sq_setup_grid(sq_ctx** out, int n1, int n2, int n3, double h, int fd_half_or
     if ((rcode = select_quad_kernels(c))) { free_ctx(c); return rcode; }
     c->red_blocks = c->sm_count * 4;
     if ((rcode = dev_alloc(&c->d_W, sizeof(double) * c->g.Nd * (npl + 1))) ||
-        (rcode = dev_alloc(&c->d_red, sizeof(double) * 3 * c->red_blocks)) ||
+        (rcode = dev_alloc(&c->d_red, sizeof(double) * RED_VALUES * c->red_blocks)) ||
         (rcode = dev_alloc(&c->d_fermi, sizeof(double) * 32)) ||
         (rcode = dev_alloc(&c->d_count, sizeof(unsigned) * 4)) || (rcode = dev_alloc(&c->d_err, sizeof(unsigned)))) {
         free_ctx(c);

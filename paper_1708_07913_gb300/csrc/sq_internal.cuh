@@ -175,7 +175,7 @@ struct sq_ctx {
     int* d_klen;
     int nl_cap;
     // quadrature weights and reductions
-    double* d_W;                     // [Nd][npl+1]
+    double* d_W;                     // [npl+1][Nd]
     double* d_red;                   // block partials
     double* d_fermi;                 // bisection state
     unsigned* d_count;               // last-block counters
@@ -197,6 +197,7 @@ int run_density(sq_ctx* ctx, const double* chi, const double* zeta, double mu, d
 int enqueue_fermi(sq_ctx* ctx, const double* chi, const double* zeta, double Ne, double kT);
 int enqueue_density(sq_ctx* ctx, const double* chi, const double* zeta, double mu, double kT, double* rho,
                     int mu_from_state);
+constexpr int RED_VALUES = 7;        // values a reduction block leaves in d_red, at most
 constexpr int FERMI_STATE = 12;      // doubles of the device Fermi/energy state
 int fermi_result(const double* st_host, double* mu, double* eb, double* es, double* ne);
 int launch_proj_tables(sq_ctx* ctx, const double* d_R);

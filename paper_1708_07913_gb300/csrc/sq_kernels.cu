@@ -131,143 +131,193 @@ int launch_support_masks(sq_ctx* ctx)
 // leading principal minors p_0 = 1, p_i = (a_i - x) p_{i-1} - b_{i-1}^2 p_{i-2}
 // (an exact zero takes the sign opposite to its predecessor).  Minors are
 // rescaled by powers of two to stay in range; no division is needed.
+//
+// FP64 bounds it (two lanes per clock and SM), so signs and exponents are read
+// from the high words and a step is left with three FP64 operations; a node has
+// two threads, one per end of the spectrum, in blocks of one warp, which also
+// spreads small grids over the SMs, and its coefficients (b squared) lie in
+// shared memory.
 // ------------------------------------------------------------------------
-__device__ int sturm_count(int k, const double* a, const double* b, double x)
+constexpr int TRI_NODES = 16;                     // nodes of a block (one warp)
+
+__device__ inline int hi_word(double v) { return __double2hiint(v); }
+
+// Eigenvalues below x; a and b2 with stride TRI_NODES.
+__device__ int sturm_count(int k, const double* a, const double* b2, double x)
 {
-    double pm = 1.0, p = a[0] - x;
-    int sprev = 1, cnt = 0;
-    int s = (p > 0.0) ? 1 : (p < 0.0 ? -1 : -sprev);
-    if (s != sprev) ++cnt;
-    sprev = s;
-    for (int i = 1; i < k; ++i) {
-        double bb = b[i - 1] * b[i - 1];
-        double pn = (a[i] - x) * p - bb * pm;
+    double pm = 1.0, p = 1.0, bb = 0.0;
+    int cnt = 0;
+    unsigned sprev = 0;                           // sign bit of the predecessor
+    for (int i = 0; i < k; ++i) {
+        const double pn = (a[i * TRI_NODES] - x) * p - bb * pm;
         pm = p;
         p = pn;
-        s = (p > 0.0) ? 1 : (p < 0.0 ? -1 : -sprev);
-        if (s != sprev) ++cnt;
+        bb = b2[i * TRI_NODES];
+        const int h = hi_word(p), m = hi_word(pm);
+        const bool zero = ((h & 0x7fffffff) | __double2loint(p)) == 0;
+        const unsigned s = zero ? sprev ^ 1u : (unsigned)h >> 31;
+        cnt += s != sprev;
         sprev = s;
-        double ap = fabs(p), am = fabs(pm);
-        if (ap > 0x1p+256 || am > 0x1p+256) { p *= 0x1p-256; pm *= 0x1p-256; }
-        else if (ap < 0x1p-256 && am < 0x1p-256) { p *= 0x1p+256; pm *= 0x1p+256; }
+        const int eh = h & 0x7fffffff, em = m & 0x7fffffff;
+        constexpr int BIG = (1023 + 256) << 20, SMALL = (1023 - 256) << 20;
+        if (eh > BIG || em > BIG) { p *= 0x1p-256; pm *= 0x1p-256; }
+        else if (eh < SMALL && em < SMALL) { p *= 0x1p+256; pm *= 0x1p+256; }
     }
     return cnt;
 }
 
-__global__ void tridiag_bounds_kernel(const double* __restrict__ alpha, const double* __restrict__ beta,
-                                      const int* __restrict__ klen, int cap, long long Nd, double margin,
-                                      double* __restrict__ chi, double* __restrict__ zeta)
+// One warp per TRI_NODES nodes: lane = node + 16 * end (0: smallest, 1: largest eigenvalue).
+__global__ void __launch_bounds__(32) tridiag_bounds_kernel(const double* __restrict__ alpha, const double* __restrict__ beta,
+                                                            const int* __restrict__ klen, int cap, long long Nd,
+                                                            double margin, double* __restrict__ chi,
+                                                            double* __restrict__ zeta)
 {
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < Nd;
-         q += (long long)gridDim.x * blockDim.x) {
+    extern __shared__ double tsm[];               // a then b^2, [cap][TRI_NODES] each
+    const int lane = threadIdx.x, n = lane & (TRI_NODES - 1), end = lane >> 4;
+    double* A = tsm + n;
+    double* B = tsm + (size_t)cap * TRI_NODES + n;
+    for (long long q0 = (long long)blockIdx.x * TRI_NODES; q0 < Nd; q0 += (long long)gridDim.x * TRI_NODES) {
+        const long long q = q0 + n < Nd ? q0 + n : Nd - 1;
+        const int k = klen[q];
         const double* a = alpha + q * cap;
         const double* b = beta + q * cap;
-        int k = klen[q];
+        __syncwarp();
         double glo = INFINITY, ghi = -INFINITY;
         for (int i = 0; i < k; ++i) {
-            double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i < k - 1 ? fabs(b[i]) : 0.0);
+            const double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i < k - 1 ? fabs(b[i]) : 0.0);
             glo = fmin(glo, a[i] - r);
             ghi = fmax(ghi, a[i] + r);
+            if (end == 0) A[i * TRI_NODES] = a[i];
+            else B[i * TRI_NODES] = i < k - 1 ? b[i] * b[i] : 0.0;
         }
-        double pad = 1e-12 * (fabs(glo) + fabs(ghi)) + 1e-300;
-        glo -= pad;
-        ghi += pad;
-        double lo = glo, hi = ghi;
+        __syncwarp();
+        const double pad = 1e-12 * (fabs(glo) + fabs(ghi)) + 1e-300;
+        double lo = glo - pad, hi = ghi + pad;
+        const int want = end == 0 ? 1 : k;
         for (int it = 0; it < 200; ++it) {
-            double mid = 0.5 * (lo + hi);
+            const double mid = 0.5 * (lo + hi);
             if (mid == lo || mid == hi) break;
-            if (sturm_count(k, a, b, mid) >= 1) hi = mid; else lo = mid;
+            if (sturm_count(k, A, B, mid) >= want) hi = mid; else lo = mid;
         }
-        double tmin = 0.5 * (lo + hi);
-        lo = glo;
-        hi = ghi;
-        for (int it = 0; it < 200; ++it) {
-            double mid = 0.5 * (lo + hi);
-            if (mid == lo || mid == hi) break;
-            if (sturm_count(k, a, b, mid) >= k) hi = mid; else lo = mid;
+        __syncwarp();
+        const double theta = 0.5 * (lo + hi), other = __shfl_xor_sync(0xffffffffu, theta, TRI_NODES);
+        if (end == 0 && q0 + n < Nd) {
+            const double tmin = theta, tmax = other;
+            const double width = fmax(tmax - tmin, 1.0);
+            const double L = tmin - margin * width, H = tmax + margin * width;
+            chi[q] = 0.5 * (H + L);
+            zeta[q] = 0.5 * (H - L);
         }
-        double tmax = 0.5 * (lo + hi);
-        double width = fmax(tmax - tmin, 1.0);
-        double L = tmin - margin * width, H = tmax + margin * width;
-        chi[q] = 0.5 * (H + L);
-        zeta[q] = 0.5 * (H - L);
     }
 }
 
 int launch_tridiag_bounds(sq_ctx* ctx, double margin, double* chi, double* zeta)
 {
-    long long Nd = ctx->g.Nd;
-    int blocks = (int)std::min<long long>((Nd + 127) / 128, (long long)ctx->sm_count * 16);
-    tridiag_bounds_kernel<<<blocks, 128, 0, ctx->stream>>>(ctx->d_alpha, ctx->d_beta, ctx->d_klen, ctx->nl_cap,
-                                                           Nd, margin, chi, zeta);
+    const long long Nd = ctx->g.Nd;
+    const int blocks = (int)std::min<long long>((Nd + TRI_NODES - 1) / TRI_NODES, (long long)ctx->sm_count * 32);
+    const size_t bytes = (size_t)2 * ctx->nl_cap * TRI_NODES * sizeof(double);      // at most 512 steps: 128 KB
+    if (bytes > 48 * 1024) {                      // raise only (see the region kernels' dispatch)
+        cudaFuncAttributes fa;
+        if (cudaFuncGetAttributes(&fa, tridiag_bounds_kernel) != cudaSuccess) return SQ_ECUDA;
+        if ((int)bytes > fa.maxDynamicSharedSizeBytes &&
+            cudaFuncSetAttribute(tridiag_bounds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
+                cudaSuccess)
+            return SQ_ECUDA;
+    }
+    tridiag_bounds_kernel<<<blocks, 32, bytes, ctx->stream>>>(ctx->d_alpha, ctx->d_beta, ctx->d_klen, ctx->nl_cap, Nd,
+                                                              margin, chi, zeta);
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
 
 // ------------------------------------------------------------------------
 // Quadrature weights (Eq. cqj by discrete orthogonality at the zeros x_k of
-// T_{npl+1}):  W_qk = (2/K) [ rho^0/2 + sum_{j>=1} rho^j T_j(x_k) ],  K = npl+1.
-// T_j(x_k) by the three-term recurrence, tabulated per block in shared memory.
+// T_{npl+1}):  W_qk = (2/K) [ rho^0/2 + sum_{j>=1} rho^j T_j(x_k) ],  K = npl+1,
+// stored zero by zero ([K][Nd]) so that the kernels with a thread per node read
+// them coalesced.  T_j(x_{K-1-k}) = (-1)^j T_j(x_k): the even and the odd part
+// of the sum serve two zeros, which halves the FP64 multiply-adds that bound
+// the kernel (two lanes per clock and SM).  A block takes 32 nodes, a lane each,
+// and its warps the zeros; T_j(x_k) from a table in shared memory, or by the three-term
+// recurrence where K x K/2 doubles do not fit.
 // ------------------------------------------------------------------------
-__global__ void weights_kernel(const double* __restrict__ mom, double* __restrict__ W, long long Nd, int K,
-                               int use_table)
+constexpr int WT_NODES = 32, WT_T = 256;
+
+__global__ void __launch_bounds__(WT_T) weights_kernel(const double* __restrict__ mom, double* __restrict__ W, long long Nd,
+                                                       int K, int use_table)
 {
-    extern __shared__ double Ttab[];   // [K][K]: Ttab[j*K + k] = T_j(x_k)
-    if (use_table) {
-        for (int k = threadIdx.x; k < K; k += blockDim.x) {
-            double x = cos(M_PI * (k + 0.5) / K);
+    extern __shared__ double wsm[];
+    const int H = (K + 1) / 2, KP = K | 1;               // odd pitch: lanes in distinct banks
+    double* r = wsm;                                     // [WT_NODES][KP] moments, rho^0 halved
+    double* T = wsm + WT_NODES * KP;                     // [H][K]: T_j(x_k)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (use_table)
+        for (int k = threadIdx.x; k < H; k += WT_T) {
+            const double x = cos(M_PI * (k + 0.5) / K);
             double tm = 1.0, t = x;
-            Ttab[k] = 1.0;
-            if (K > 1) Ttab[K + k] = x;
+            T[k * K] = 1.0;
+            T[k * K + 1] = x;
             for (int j = 2; j < K; ++j) {
-                double tn = 2.0 * x * t - tm;
+                const double tn = 2.0 * x * t - tm;
                 tm = t;
                 t = tn;
-                Ttab[j * K + k] = t;
+                T[k * K + j] = t;
             }
+        }
+    const double c = 2.0 / K;
+    for (long long q0 = (long long)blockIdx.x * WT_NODES; q0 < Nd; q0 += (long long)gridDim.x * WT_NODES) {
+        const int nq = (int)(Nd - q0 < WT_NODES ? Nd - q0 : WT_NODES);
+        __syncthreads();
+        for (int i = threadIdx.x; i < nq * K; i += WT_T) {
+            const int n = i / K, j = i - n * K;
+            const double v = mom[q0 * K + i];
+            r[n * KP + j] = j == 0 ? 0.5 * v : v;
         }
         __syncthreads();
-    }
-    const long long tot = Nd * K;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < tot;
-         idx += (long long)gridDim.x * blockDim.x) {
-        long long q = idx / K;
-        int k = (int)(idx % K);
-        const double* r = mom + q * K;
-        double s = 0.5 * r[0];
-        if (use_table) {
-            for (int j = 1; j < K; ++j) s += r[j] * Ttab[j * K + k];
-        } else {
-            double x = cos(M_PI * (k + 0.5) / K);
-            double tm = 1.0, t = x;
-            for (int j = 1; j < K; ++j) {
-                s += r[j] * t;
-                double tn = 2.0 * x * t - tm;
-                tm = t;
-                t = tn;
+        if (lane < nq) {
+            const double* rn = r + lane * KP;
+            for (int k = warp; k < H; k += WT_T / 32) {
+                double e = rn[0], o = 0.0;
+                if (use_table) {
+                    const double* Tk = T + k * K;
+                    int j = 1;
+                    for (; j + 1 < K; j += 2) {
+                        o += rn[j] * Tk[j];
+                        e += rn[j + 1] * Tk[j + 1];
+                    }
+                    if (j < K) o += rn[j] * Tk[j];
+                } else {
+                    const double x = cos(M_PI * (k + 0.5) / K);
+                    double tm = 1.0, t = x;
+                    for (int j = 1; j < K; ++j) {
+                        if (j & 1) o += rn[j] * t;
+                        else e += rn[j] * t;
+                        const double tn = 2.0 * x * t - tm;
+                        tm = t;
+                        t = tn;
+                    }
+                }
+                W[(long long)k * Nd + q0 + lane] = c * (e + o);
+                if (K - 1 - k != k) W[(long long)(K - 1 - k) * Nd + q0 + lane] = c * (e - o);
             }
         }
-        W[idx] = 2.0 / K * s;
     }
 }
 
 int launch_weights(sq_ctx* ctx, const double* moments)
 {
-    int K = ctx->npl + 1;
-    long long tot = ctx->g.Nd * K;
-    size_t tbytes = (size_t)K * K * sizeof(double);
-    int use_table = tbytes <= 96 * 1024;
-    if (use_table && tbytes > 48 * 1024) {        // raise only (see the region kernels' dispatch)
+    const int K = ctx->npl + 1, H = (K + 1) / 2;
+    const size_t rows = (size_t)WT_NODES * (K | 1) * sizeof(double), table = (size_t)H * K * sizeof(double);
+    const int use_table = rows + table <= 100 * 1024;
+    const size_t bytes = rows + (use_table ? table : 0);
+    if (bytes > 48 * 1024) {                      // raise only (see the region kernels' dispatch)
         cudaFuncAttributes fa;
         if (cudaFuncGetAttributes(&fa, weights_kernel) != cudaSuccess) return SQ_ECUDA;
-        if ((int)tbytes > fa.maxDynamicSharedSizeBytes &&
-            cudaFuncSetAttribute(weights_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tbytes) !=
-                cudaSuccess)
+        if ((int)bytes > fa.maxDynamicSharedSizeBytes &&
+            cudaFuncSetAttribute(weights_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
             return SQ_ECUDA;
     }
-    int blocks = (int)std::min<long long>((tot + 255) / 256, (long long)ctx->sm_count * 8);
-    weights_kernel<<<blocks, 256, use_table ? tbytes : 0, ctx->stream>>>(moments, ctx->d_W, ctx->g.Nd, K,
-                                                                         use_table);
+    const int blocks = (int)std::min<long long>((ctx->g.Nd + WT_NODES - 1) / WT_NODES, (long long)ctx->sm_count * 4);
+    weights_kernel<<<blocks, WT_T, bytes, ctx->stream>>>(moments, ctx->d_W, ctx->g.Nd, K, use_table);
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
@@ -305,46 +355,72 @@ __device__ inline void block_reduce(double (&v)[NV], double* sh)
     }
 }
 
-// Fermi state layout (doubles)
-enum { F_LO = 0, F_HI, F_NE, F_KT, F_NLO, F_NHI, F_DONE, F_ITERS, F_STATUS, F_EB, F_ES, F_NEL, F_NSTATE };
-static_assert(F_NSTATE == FERMI_STATE, "Fermi state size");
+// Fermi state (doubles): the first FERMI_STATE are read by the host.
+enum { F_LO = 0, F_HI, F_NE, F_KT, F_NLO, F_NHI, F_DONE, F_ITERS, F_STATUS, F_EB, F_ES, F_NEL, F_NSTATE,
+       F_FINE = 12, F_NPTS, F_PTS };
+constexpr int FERMI_PTS = 7;
+static_assert(F_NSTATE == FERMI_STATE && F_PTS + FERMI_PTS <= 32, "Fermi state size");
 
-// min(chi - zeta) - 10 kT and max(chi + zeta) + 10 kT
+// Sum of one value per thread over the partials of all blocks, by the whole of
+// the last block in a fixed order; valid in thread 0.
+template <int NV>
+__device__ inline void sum_partials(const double* red, unsigned nb, double (&v)[NV], double* sh)
+{
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+        v[i] = 0.0;
+        for (unsigned b = threadIdx.x; b < nb; b += blockDim.x) v[i] += __ldcg(red + (size_t)NV * b + i);
+    }
+    __syncthreads();
+    block_reduce<NV>(v, sh);
+}
+
+// min(chi - zeta) - 10 kT and max(chi + zeta) + 10 kT; the ends are the first points of the search.
 __global__ void fermi_bracket_kernel(const double* __restrict__ chi, const double* __restrict__ zeta, long long Nd,
                                      double* red, unsigned* count, double* st)
 {
     __shared__ double sh[64];
     __shared__ bool last;
     double lo = INFINITY, hi = -INFINITY;
+    auto block_minmax = [&]() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        if ((threadIdx.x & 31) == 0) { sh[threadIdx.x >> 5] = lo; sh[32 + (threadIdx.x >> 5)] = hi; }
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) { lo = fmin(lo, sh[k]); hi = fmax(hi, sh[32 + k]); }
+    };
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < Nd;
          q += (long long)gridDim.x * blockDim.x) {
         lo = fmin(lo, chi[q] - zeta[q]);
         hi = fmax(hi, chi[q] + zeta[q]);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    if ((threadIdx.x & 31) == 0) { sh[threadIdx.x >> 5] = lo; sh[32 + (threadIdx.x >> 5)] = hi; }
-    __syncthreads();
+    block_minmax();
     if (threadIdx.x == 0) {
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) { lo = fmin(lo, sh[k]); hi = fmax(hi, sh[32 + k]); }
         red[2 * blockIdx.x] = lo;
         red[2 * blockIdx.x + 1] = hi;
         __threadfence();
         last = atomicAdd(count, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (last && threadIdx.x == 0) {
-        __threadfence();
-        double L = INFINITY, H = -INFINITY;
-        for (unsigned b = 0; b < gridDim.x; ++b) {
-            L = fmin(L, ((volatile double*)red)[2 * b]);
-            H = fmax(H, ((volatile double*)red)[2 * b + 1]);
-        }
-        st[F_LO] = L - 10.0 * st[F_KT];
-        st[F_HI] = H + 10.0 * st[F_KT];
+    if (!last) return;
+    __threadfence();
+    lo = INFINITY;
+    hi = -INFINITY;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+        lo = fmin(lo, __ldcg(red + 2 * b));
+        hi = fmax(hi, __ldcg(red + 2 * b + 1));
+    }
+    __syncthreads();
+    block_minmax();
+    if (threadIdx.x == 0) {
+        st[F_LO] = st[F_PTS] = lo - 10.0 * st[F_KT];
+        st[F_HI] = st[F_PTS + 1] = hi + 10.0 * st[F_KT];
+        st[F_NPTS] = 2.0;
+        st[F_FINE] = -1.0;                                // the ends come first
         st[F_DONE] = 0.0;
         st[F_ITERS] = 0.0;
         st[F_STATUS] = 0.0;
@@ -352,70 +428,183 @@ __global__ void fermi_bracket_kernel(const double* __restrict__ chi, const doubl
     }
 }
 
-// Electron count N(mu) = 2 sum_q sum_k W_qk g((chi_q + zeta_q x_k - mu)/kT).
-// mode 0: N(lo); mode 1: N(hi) and bracket check; mode 2: one bisection step.
-__global__ void fermi_count_kernel(const double* __restrict__ W, const double* __restrict__ chi,
-                                   const double* __restrict__ zeta, long long Nd, int K, int mode, double* red,
-                                   unsigned* count, double* st)
+// First zero k with chi + zeta x_k - mu <= 41 kT, or up to two before it (x_k
+// falls with k, FP32, the margin covers its rounding): where the terms begin
+// that are not 0.  With the sign of the bound turned, past which they are 1.
+__device__ inline int zero_index(double c, double z, double bound, int K, bool up)
 {
-    __shared__ double sh[32];
-    __shared__ bool last;
-    const double lo = st[F_LO], hi = st[F_HI], kT = st[F_KT];
-    double mu;
-    if (mode == 0) mu = lo;
-    else if (mode == 1) mu = hi;
-    else {
-        if (st[F_DONE] != 0.0) return;                 // uniform over the grid
-        mu = 0.5 * (lo + hi);
-        if (mu == lo || mu == hi) {                    // converged in FP64
-            if (blockIdx.x == 0 && threadIdx.x == 0) st[F_DONE] = 1.0;
-            return;
-        }
+    const float x = fminf(1.0f, fmaxf(-1.0f, (float)(bound - c) / (float)z));
+    const float k = acosf(x) * (float)K * 0.318309886f - 0.5f;
+    const int i = up ? (int)ceilf(k) + 1 : (int)floorf(k) - 1;
+    return min(K, max(0, i));
+}
+
+// The next points of the search (thread 0).  lo < hi bracket the electron
+// count, fl and fh the counts there.
+__device__ void fermi_next(double* st, double lo, double hi, double fl, double fh, int coarse)
+{
+    const double mid = 0.5 * (lo + hi), w = hi - lo, kT = st[F_KT];
+    st[F_LO] = lo;
+    st[F_HI] = hi;
+    st[F_NLO] = fl;
+    st[F_NHI] = fh;
+    double p[FERMI_PTS];
+    int n = 0;
+    const double tiny = 8.0 * 2.220446049250313e-16 * fmax(fabs(lo), fabs(hi));
+    if (mid == lo || mid == hi) {                         // adjacent in FP64
+        st[F_DONE] = 1.0;
+        return;
     }
-    __shared__ double xk[MAX_NPL + 1];
+    const bool fine = w < 0.25 * kT;
+    if (!fine && coarse == 1) {
+        p[n++] = mid;
+    } else if (!fine || w <= 8.0 * tiny) {                // two or three levels of bisection at once
+        const double a = 0.5 * (lo + mid), b = 0.5 * (mid + hi);
+        if (fine) p[n++] = 0.5 * (lo + a);
+        p[n++] = a;
+        if (fine) p[n++] = 0.5 * (a + mid);
+        p[n++] = mid;
+        if (fine) p[n++] = 0.5 * (mid + b);
+        p[n++] = b;
+        if (fine) p[n++] = 0.5 * (b + hi);
+    } else {                                              // the count is smooth on the scale kT: around the secant
+        const double x = lo + w * ((st[F_NE] - fl) / (fh - fl));
+        const double d = 0.25 * w * (w / kT) + 0.25 * tiny;
+        const double off[6] = {-8.0 * d, -d, 0.0, d, 8.0 * d, mid - x};
+        for (int i = 0; i < 6; ++i) {
+            const double v = x + off[i];
+            if (v > lo && v < hi) p[n++] = v;
+        }
+        if (n == 0) p[n++] = mid;
+        for (int i = 1; i < n; ++i)                       // ascending
+            for (int j = i; j > 0 && p[j] < p[j - 1]; --j) {
+                const double t = p[j];
+                p[j] = p[j - 1];
+                p[j - 1] = t;
+            }
+    }
+    for (int i = 0; i < n; ++i) st[F_PTS + i] = p[i];
+    st[F_NPTS] = (double)n;
+    st[F_FINE] = fine ? 1.0 : 0.0;
+}
+
+// Electron count N(mu) = 2 sum_q sum_k W_qk g((chi_q + zeta_q x_k - mu)/kT) at
+// up to FERMI_PTS points at once, then (last block) the bracket they leave and
+// the next points.  Beyond |t| = 40 the Fermi factor is 1.0 exactly in FP64
+// (t < -40) or below 4.3e-18 (t > 40, dropped: < 1e-16 of any count here), so a
+// node visits only the zeros around mu.  What bounds it is FP64 (two lanes per
+// clock and SM): a term is an exponential and a division; within a bracket far
+// narrower than kT the points share the exponential, e^{(E-mu)/kT} = a s.  The
+// level, density and energies of 64^3 nodes at n_pl 48 took 31.8 ms with about
+// 60 bisection passes that each visited every zero, one node's row per thread,
+// and take 7.5 ms now.
+__global__ void fermi_search_kernel(const double* __restrict__ W, const double* __restrict__ chi,
+                                    const double* __restrict__ zeta, long long Nd, int K, int coarse, double* red,
+                                    unsigned* count, double* st)
+{
+    __shared__ double sh[FERMI_PTS * 32];
+    __shared__ bool last;
+    __shared__ double xk[MAX_NPL + 1], pts[FERMI_PTS], sc[FERMI_PTS];
+    if (st[F_DONE] != 0.0) return;                        // uniform over the grid
+    const double kT = st[F_KT];
+    const int np = (int)st[F_NPTS];
+    const bool fine = st[F_FINE] > 0.5;
+    const double ref = st[F_PTS + (np >> 1)];
     for (int k = threadIdx.x; k < K; k += blockDim.x) xk[k] = cos(M_PI * (k + 0.5) / K);
+    if ((int)threadIdx.x < np) {
+        pts[threadIdx.x] = st[F_PTS + threadIdx.x];
+        sc[threadIdx.x] = fine ? exp((ref - st[F_PTS + threadIdx.x]) / kT) : 0.0;
+    }
     __syncthreads();
-    double acc[1] = {0.0};
+    double acc[FERMI_PTS];
+#pragma unroll
+    for (int i = 0; i < FERMI_PTS; ++i) acc[i] = 0.0;
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < Nd;
          q += (long long)gridDim.x * blockDim.x) {
         const double c = chi[q], z = zeta[q];
-        const double* w = W + q * K;
-        double s = 0.0;
-        for (int k = 0; k < K; ++k) {
-            double t = (c + z * xk[k] - mu) / kT;
-            // beyond |t| = 40 the Fermi factor is 1.0 exactly in FP64 (t < -40)
-            // or below 4.3e-18 (t > 40, dropped: < 1e-16 of any count here)
-            if (t > 40.0) continue;
-            s += (t < -40.0) ? w[k] : w[k] / (1.0 + exp(t));
+        const double* w = W + q;
+        if (fine) {
+            const int ka = zero_index(c, z, pts[np - 1] + 41.0 * kT, K, false);
+            const int kb = zero_index(c, z, pts[0] - 41.0 * kT, K, true);
+            double s[FERMI_PTS], full = 0.0;
+#pragma unroll
+            for (int i = 0; i < FERMI_PTS; ++i) s[i] = 0.0;
+            for (int k = ka; k < kb; ++k) {
+                const double wk = w[(long long)k * Nd], a = exp((c + z * xk[k] - ref) / kT);
+#pragma unroll
+                for (int i = 0; i < FERMI_PTS; ++i)
+                    if (i < np) s[i] += wk / (1.0 + a * sc[i]);
+            }
+            for (int k = max(ka, kb); k < K; ++k) full += w[(long long)k * Nd];
+#pragma unroll
+            for (int i = 0; i < FERMI_PTS; ++i)
+                if (i < np) acc[i] += 2.0 * (s[i] + full);
+        } else {
+#pragma unroll
+            for (int i = 0; i < FERMI_PTS; ++i) {
+                if (i >= np) break;
+                const double mu = pts[i];
+                const int ka = zero_index(c, z, mu + 41.0 * kT, K, false);
+                const int kb = zero_index(c, z, mu - 41.0 * kT, K, true);
+                double s = 0.0;
+                for (int k = ka; k < kb; ++k) {
+                    const double t = (c + z * xk[k] - mu) / kT;
+                    if (t > 40.0) continue;
+                    const double wk = w[(long long)k * Nd];
+                    s += (t < -40.0) ? wk : wk / (1.0 + exp(t));
+                }
+                for (int k = max(ka, kb); k < K; ++k) s += w[(long long)k * Nd];
+                acc[i] += 2.0 * s;
+            }
         }
-        acc[0] += 2.0 * s;
     }
-    block_reduce<1>(acc, sh);
+    block_reduce<FERMI_PTS>(acc, sh);
     if (threadIdx.x == 0) {
-        red[blockIdx.x] = acc[0];
+        for (int i = 0; i < FERMI_PTS; ++i) red[(size_t)FERMI_PTS * blockIdx.x + i] = acc[i];
         __threadfence();
         last = atomicAdd(count, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (last && threadIdx.x == 0) {
-        __threadfence();
-        double N = 0.0;
-        for (unsigned b = 0; b < gridDim.x; ++b) N += ((volatile double*)red)[b];
-        const double Ne = st[F_NE];
-        if (mode == 0) st[F_NLO] = N;
-        else if (mode == 1) {
-            st[F_NHI] = N;
-            if (!(st[F_NLO] <= Ne && N >= Ne)) { st[F_STATUS] = (double)SQ_ENOCONV; st[F_DONE] = 1.0; }
-        } else {
-            if (N < Ne) st[F_LO] = mu; else st[F_HI] = mu;
-            st[F_ITERS] += 1.0;
-            if (st[F_ITERS] >= 200.0) st[F_DONE] = 1.0;
+    if (!last) return;
+    __threadfence();
+    sum_partials<FERMI_PTS>(red, gridDim.x, acc, sh);
+    if (threadIdx.x != 0) return;
+    const double Ne = st[F_NE];
+    *count = 0;
+    if (st[F_FINE] < -0.5) {                              // the ends
+        if (!(acc[0] <= Ne && acc[1] >= Ne)) {
+            st[F_NLO] = acc[0];
+            st[F_NHI] = acc[1];
+            st[F_STATUS] = (double)SQ_ENOCONV;
+            st[F_DONE] = 1.0;
+            return;
         }
-        *count = 0;
+        fermi_next(st, st[F_LO], st[F_HI], acc[0], acc[1], coarse);
+        return;
     }
+    double lo = st[F_LO], hi = st[F_HI], fl = st[F_NLO], fh = st[F_NHI];
+    // three points of one bisection tree (coarse) are walked as bisection walks them; else the first rise past Ne
+    if (!fine && np == 3) {
+        const int i = acc[1] < Ne ? 2 : 0;
+        if (i == 2) { lo = pts[1]; fl = acc[1]; } else { hi = pts[1]; fh = acc[1]; }
+        if (acc[i] < Ne) { lo = pts[i]; fl = acc[i]; } else { hi = pts[i]; fh = acc[i]; }
+    } else {
+        for (int i = 0; i < np; ++i) {
+            if (acc[i] < Ne) {
+                lo = pts[i];
+                fl = acc[i];
+            } else {
+                hi = pts[i];
+                fh = acc[i];
+                break;
+            }
+        }
+    }
+    st[F_ITERS] += 1.0;
+    fermi_next(st, lo, hi, fl, fh, coarse);
 }
 
-// Bisection state reset (a kernel rather than a host copy, so the whole
+// Search state reset (a kernel rather than a host copy, so the whole
 // Fermi-level search can be captured in a CUDA graph).
 __global__ void fermi_init_kernel(double* st, double Ne, double kT)
 {
@@ -426,38 +615,61 @@ __global__ void fermi_init_kernel(double* st, double Ne, double kT)
     }
 }
 
+// Blocks of 256 threads where that fills the GPU, else of 64, so that small systems spread over the SMs.
+static int node_threads(long long Nd, int sm_count) { return Nd >= (long long)sm_count * 512 ? RED_T : 64; }
+static int node_blocks(const sq_ctx* ctx, int threads)
+{
+    return (int)std::min<long long>((ctx->g.Nd + threads - 1) / threads, ctx->red_blocks);
+}
+
+static int enqueue_search(sq_ctx* ctx, const double* chi, const double* zeta, int launches)
+{
+    const int T = node_threads(ctx->g.Nd, ctx->sm_count), B = node_blocks(ctx, T);
+    // far from the level a large system takes one point per pass (FP64-bound), a small one three (launch-bound)
+    const int coarse = ctx->g.Nd >= 65536 ? 1 : 3;
+    for (int it = 0; it < launches; ++it)
+        fermi_search_kernel<<<B, T, 0, ctx->stream>>>(ctx->d_W, chi, zeta, ctx->g.Nd, ctx->npl + 1, coarse, ctx->d_red,
+                                                      ctx->d_count, ctx->d_fermi);
+    ctx->launches += launches;
+    return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
+}
+
+static int enqueue_search_start(sq_ctx* ctx, const double* chi, const double* zeta, double Ne, double kT)
+{
+    const int T = node_threads(ctx->g.Nd, ctx->sm_count);
+    fermi_init_kernel<<<1, 32, 0, ctx->stream>>>(ctx->d_fermi, Ne, kT);
+    fermi_bracket_kernel<<<node_blocks(ctx, T), T, 0, ctx->stream>>>(chi, zeta, ctx->g.Nd, ctx->d_red, ctx->d_count,
+                                                                     ctx->d_fermi);
+    ctx->launches += 2;
+    return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
+}
+
+// Passes that always end the search: bisection alone to kT/4 (at most 1e9 times
+// narrower than the spectrum for one point per pass) and to the last bit of FP64
+// after that; the passes past its end return at once.
+constexpr int FERMI_PASSES = 56, FERMI_FIRST = 18;
+
 // Enqueue the whole Fermi-level search on ctx->stream (no host wait); the
 // result stays in the device state: mu = (st[F_LO] + st[F_HI]) / 2, status
 // in st[F_STATUS].
 int enqueue_fermi(sq_ctx* ctx, const double* chi, const double* zeta, double Ne, double kT)
 {
-    const long long Nd = ctx->g.Nd;
-    const int K = ctx->npl + 1;
-    fermi_init_kernel<<<1, 32, 0, ctx->stream>>>(ctx->d_fermi, Ne, kT);
-    ctx->launches++;
-    const int blocks = ctx->red_blocks;
-    fermi_bracket_kernel<<<blocks, RED_T, 0, ctx->stream>>>(chi, zeta, Nd, ctx->d_red, ctx->d_count, ctx->d_fermi);
-    fermi_count_kernel<<<blocks, RED_T, 0, ctx->stream>>>(ctx->d_W, chi, zeta, Nd, K, 0, ctx->d_red, ctx->d_count,
-                                                         ctx->d_fermi);
-    fermi_count_kernel<<<blocks, RED_T, 0, ctx->stream>>>(ctx->d_W, chi, zeta, Nd, K, 1, ctx->d_red, ctx->d_count,
-                                                         ctx->d_fermi);
-    ctx->launches += 3;
-    for (int it = 0; it < 201; ++it) {
-        fermi_count_kernel<<<blocks, RED_T, 0, ctx->stream>>>(ctx->d_W, chi, zeta, Nd, K, 2, ctx->d_red,
-                                                             ctx->d_count, ctx->d_fermi);
-        ctx->launches++;
-    }
-    SQ_CUDA_TRY(cudaGetLastError());
-    return SQ_OK;
+    const int rc = enqueue_search_start(ctx, chi, zeta, Ne, kT);
+    return rc ? rc : enqueue_search(ctx, chi, zeta, FERMI_PASSES);
 }
 
 int run_fermi(sq_ctx* ctx, const double* chi, const double* zeta, double Ne, double kT, double* mu)
 {
-    int rc = enqueue_fermi(ctx, chi, zeta, Ne, kT);
+    int rc = enqueue_search_start(ctx, chi, zeta, Ne, kT);
     if (rc) return rc;
     double st[F_NSTATE];
-    SQ_CUDA_TRY(cudaMemcpyAsync(st, ctx->d_fermi, sizeof(st), cudaMemcpyDeviceToHost, ctx->stream));
-    SQ_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+    for (int done = 0, n = FERMI_FIRST; done < FERMI_PASSES; done += n) {     // most searches end in the first lot
+        n = std::min(n, FERMI_PASSES - done);
+        if ((rc = enqueue_search(ctx, chi, zeta, n))) return rc;
+        SQ_CUDA_TRY(cudaMemcpyAsync(st, ctx->d_fermi, sizeof(st), cudaMemcpyDeviceToHost, ctx->stream));
+        SQ_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        if (st[F_DONE] != 0.0) break;
+    }
     if (st[F_STATUS] != 0.0) return (int)st[F_STATUS];
     *mu = 0.5 * (st[F_LO] + st[F_HI]);
     return SQ_OK;
@@ -490,28 +702,32 @@ __global__ void density_kernel(const double* __restrict__ W, const double* __res
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < Nd;
          q += (long long)gridDim.x * blockDim.x) {
         const double c = chi[q], z = zeta[q];
-        const double* w = W + q * K;
+        const double* w = W + q;
+        const int ka = zero_index(c, z, mu + 41.0 * kT, K, false), kb = zero_index(c, z, mu - 41.0 * kT, K, true);
         double r = 0.0, eb = 0.0, es = 0.0;
-        for (int k = 0; k < K; ++k) {
-            double E = c + z * xk[k];
-            double t = (E - mu) / kT;
+        for (int k = ka; k < kb; ++k) {
+            const double E = c + z * xk[k];
+            const double t = (E - mu) / kT;
             if (t > 40.0) continue;                    // g < 4.3e-18: no density, energy or entropy
-            double wk = w[k];
+            const double wk = w[(long long)k * Nd];
             if (t < -40.0) {                           // g == 1.0 exactly in FP64, entropy term 0
                 r += wk;
                 eb += 2.0 * wk * E;
                 continue;
             }
-            double g = 1.0 / (1.0 + exp(t));
-            double gm = 1.0 / (1.0 + exp(-t));
+            // e = e^{-|t|}: g = 1/(1+e) or e/(1+e), and -(g ln g + (1-g) ln(1-g)) = ln(1+e) + |t| e/(1+e)
+            const double e = exp(-fabs(t)), d = 1.0 / (1.0 + e), small = e * d;
+            const double g = t > 0.0 ? small : d;
             r += wk * g;
             eb += 2.0 * wk * E * g;
-            double sf = 0.0;
-            if (g > 0.0) sf += g * log(g);
-            if (gm > 0.0) sf += gm * log(gm);
-            es += 2.0 * kT * wk * sf;
+            es -= 2.0 * kT * wk * (log1p(e) + fabs(t) * small);
         }
-        double rq = 2.0 / h3 * r;
+        for (int k = max(ka, kb); k < K; ++k) {        // the rest below mu - 40 kT
+            const double wk = w[(long long)k * Nd];
+            r += wk;
+            eb += 2.0 * wk * (c + z * xk[k]);
+        }
+        const double rq = 2.0 / h3 * r;
         rho[q] = rq;
         acc[0] += eb;
         acc[1] += es;
@@ -526,17 +742,13 @@ __global__ void density_kernel(const double* __restrict__ W, const double* __res
         last = atomicAdd(count, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (last && threadIdx.x == 0) {
-        __threadfence();
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-        for (unsigned b = 0; b < gridDim.x; ++b) {
-            s0 += ((volatile double*)red)[3 * b + 0];
-            s1 += ((volatile double*)red)[3 * b + 1];
-            s2 += ((volatile double*)red)[3 * b + 2];
-        }
-        st[F_EB] = s0;
-        st[F_ES] = s1;
-        st[F_NEL] = s2;
+    if (!last) return;
+    __threadfence();
+    sum_partials<3>(red, gridDim.x, acc, sh);
+    if (threadIdx.x == 0) {
+        st[F_EB] = acc[0];
+        st[F_ES] = acc[1];
+        st[F_NEL] = acc[2];
         *count = 0;
     }
 }
@@ -544,10 +756,9 @@ __global__ void density_kernel(const double* __restrict__ W, const double* __res
 int enqueue_density(sq_ctx* ctx, const double* chi, const double* zeta, double mu, double kT, double* rho,
                     int mu_from_state)
 {
-    const int blocks = ctx->red_blocks;
-    density_kernel<<<blocks, RED_T, 0, ctx->stream>>>(ctx->d_W, chi, zeta, ctx->g.Nd, ctx->npl + 1, mu, kT,
-                                                     ctx->g.h, rho, ctx->d_red, ctx->d_count, ctx->d_fermi,
-                                                     mu_from_state);
+    const int T = node_threads(ctx->g.Nd, ctx->sm_count);
+    density_kernel<<<node_blocks(ctx, T), T, 0, ctx->stream>>>(ctx->d_W, chi, zeta, ctx->g.Nd, ctx->npl + 1, mu, kT, ctx->g.h,
+                                                               rho, ctx->d_red, ctx->d_count, ctx->d_fermi, mu_from_state);
     ctx->launches++;
     SQ_CUDA_TRY(cudaGetLastError());
     return SQ_OK;
