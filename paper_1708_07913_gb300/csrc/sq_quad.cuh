@@ -198,29 +198,64 @@ __device__ __forceinline__ void tm_sync()
 // Sum of one float per thread over the CTA: compensated FP32 trees (value and
 // running error) within the warps and then over their 16 results, so that FP64,
 // two lanes per clock on this part, is left with one addition per sum.  Every
-// warp calls quad_warp_sum before the barrier; quad_cta_sum after it, by the
-// whole of one warp, returns the total in every lane.
-__device__ __forceinline__ void two_sum_xor(float& s, float& c, int o)
+// warp calls quad_warp_sums before the barrier; quad_cta_sums after it, by the
+// whole of one warp, leaves the totals in its lane 0.
+template <int N>
+__device__ __forceinline__ void quad_warp_sums(const float (&v)[N], float2 (*red)[QD_NW])
 {
-    const float t = __shfl_xor_sync(0xffffffffu, s, o), tc = __shfl_xor_sync(0xffffffffu, c, o);
-    float e;
-    two_sum(s, t, s, e);
-    c = c + (tc + e);
-}
-__device__ __forceinline__ void quad_warp_sum(float v, float2* red)
-{
-    float s = v, c = 0.f;
+    float s[N], c[N];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) two_sum_xor(s, c, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(s, c);
-}
-__device__ __forceinline__ double quad_cta_sum(const float2* red)
-{
-    const float2 r = red[threadIdx.x & 15];
-    float s = r.x, c = r.y;
+    for (int i = 0; i < N; ++i) {
+        s[i] = v[i];
+        c[i] = 0.f;
+    }
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) two_sum_xor(s, c, o);
-    return (double)s + (double)c;
+    for (int o = 16; o > 0; o >>= 1) {
+        float t[N], tc[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {                     // the trees side by side
+            t[i] = __shfl_xor_sync(0xffffffffu, s[i], o);
+            tc[i] = __shfl_xor_sync(0xffffffffu, c[i], o);
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            float e;
+            two_sum(s[i], t[i], s[i], e);
+            c[i] = c[i] + (tc[i] + e);
+        }
+    }
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int i = 0; i < N; ++i) red[i][threadIdx.x >> 5] = make_float2(s[i], c[i]);
+}
+template <int N>
+__device__ __forceinline__ void quad_cta_sums(const float2 (*red)[QD_NW], double (&out)[N])
+{
+    float s[N], c[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const float2 r = red[i][threadIdx.x & 15];
+        s[i] = r.x;
+        c[i] = r.y;
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+        float t[N], tc[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            t[i] = __shfl_xor_sync(0xffffffffu, s[i], o);
+            tc[i] = __shfl_xor_sync(0xffffffffu, c[i], o);
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            float e;
+            two_sum(s[i], t[i], s[i], e);
+            c[i] = c[i] + (tc[i] + e);
+        }
+    }
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int i = 0; i < N; ++i) out[i] = (double)s[i] + (double)c[i];
 }
 
 // Streamed global loads that leave the L1 to the tables.
@@ -407,7 +442,7 @@ __device__ int quad_setup(const QuadArgs& a, const QuadCta<M>& k, int qi, int qj
         k.yt[i] = make_float4(in0 ? Gt[j0] : 0.f, in0 ? Dt[j0] : 0.f, in1 ? Gt[j1] : 0.f, in1 ? Dt[j1] : 0.f);
     }
     // lists: every thread its own (quad, row pair), a warp every fourth pair of planes; per pair the candidates
-    // that meet it and the warp's quads, in order, four candidates' support rows in flight
+    // that meet it and the warp's quads, in order, six candidates' support rows in flight
     {
         const uint2 none = quad_none<M>(k);
         const uint32_t xb = none.x & 0x3fff0u, yb = (none.x >> 14) & 0x3fff0u, bb = (none.y << 2) & 0x3fff0u;
@@ -427,10 +462,10 @@ __device__ int quad_setup(const QuadArgs& a, const QuadCta<M>& k, int qi, int qj
                 }
                 unsigned set = __ballot_sync(0xffffffffu, hit);
                 while (set) {                             // warp-uniform
-                    int cc[4];
-                    uint32_t m[4][4];
+                    int cc[6];
+                    uint32_t m[6][4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
+                    for (int i = 0; i < 6; ++i) {
                         cc[i] = set ? cb + __ffs(set) - 1 : -1;
                         set &= set - 1;
                         m[i][0] = m[i][1] = m[i][2] = m[i][3] = 0;
@@ -447,7 +482,7 @@ __device__ int quad_setup(const QuadArgs& a, const QuadCta<M>& k, int qi, int qj
                         if (r1 && p1) m[i][3] = src[lb + 1];
                     }
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
+                    for (int i = 0; i < 6; ++i) {
                         if (cc[i] < 0) break;
                         const int4 cr = k.cand[cc[i]];
                         const int sh = 4 * k.q - cr.y;        // region column 4q is box column sh
@@ -510,7 +545,10 @@ __device__ int quad_setup(const QuadArgs& a, const QuadCta<M>& k, int qi, int qj
                 if (rr < nrows) {
                     const int dk = (rr * inv) >> 16;          // rr / nj, exact for rr < 1024 and nj <= 32
                     const int jj = j0 + rr - dk * nj, kk = k0 + dk;
-                    ok[i] = nl_row_interval<float, M>(nl, cr.x, cr.y, jj, kk, xlo[i], xhi[i]);
+                    const uint32_t mk = a.mask[((size_t)cr.x * lb + kk) * lb + jj];
+                    xlo[i] = max(cr.y + __ffs(mk) - 1, 0);
+                    xhi[i] = min(cr.y + 31 - __clz(mk), G::S - 1);
+                    ok[i] = mk != 0 && xlo[i] <= xhi[i];
                     off[i] = (cr.w + kk) * G::PL + G::row(cr.z + jj);
                     gy[i] = Gt[lb + jj];
                     dgy[i] = Dt[lb + jj];
@@ -991,9 +1029,13 @@ __device__ void quad_sweep(const QuadArgs& a, const QuadCta<M>& k, uint32_t ca, 
     } else {
         quad_stencil<M, TT, true>(a, k, ca, cb, s, sum, centre);
     }
-    quad_warp_sum(lo2(sum.aa) + hi2(sum.aa), red[0]);
-    quad_warp_sum(lo2(sum.ab) + hi2(sum.ab), red[1]);
-    if (TT) quad_warp_sum(lo2(sum.ac) + hi2(sum.ac), red[2]);
+    if (TT) {
+        const float v[3] = {lo2(sum.aa) + hi2(sum.aa), lo2(sum.ab) + hi2(sum.ab), lo2(sum.ac) + hi2(sum.ac)};
+        quad_warp_sums<3>(v, red);
+    } else {
+        const float v[2] = {lo2(sum.aa) + hi2(sum.aa), lo2(sum.ab) + hi2(sum.ab)};
+        quad_warp_sums<2>(v, red);
+    }
     tm_sync();
 }
 
@@ -1081,10 +1123,11 @@ __device__ void quad_moments_node(const QuadArgs& a, unsigned char* smem, uint32
         const float s = s_scale[i == 0 ? 1 : 2];
         quad_sweep<M, false>(a, k, ca, cb, s, ncand, red, &s_mom[i + 1]);
         if (warp == QD_NW - 1) {                          // one with the fewest planes
-            const double d2 = quad_cta_sum(red[0]), d1 = quad_cta_sum(red[1]);
+            double d[2];
+            quad_cta_sums<2>(red, d);
             if (lane == 0) {
-                s_d2[i + 1] = d2;                         // t^{i+1} . t^{i+1}
-                s_d1[i + 1] = d1;                         // t^{i+1} . t^i
+                s_d2[i + 1] = d[0];                       // t^{i+1} . t^{i+1}
+                s_d1[i + 1] = d[1];                       // t^{i+1} . t^i
             }
             __syncwarp();
         }
@@ -1154,8 +1197,10 @@ __device__ void quad_lanczos_node(const QuadArgs& a, unsigned char* smem, uint32
             bprev = b;
         };
         if (warp == 0) {
-            const double al = quad_cta_sum(red[1]), w2 = quad_cta_sum(red[0]), v2 = quad_cta_sum(red[2]);
+            double d[3];
+            quad_cta_sums<3>(red, d);
             if (lane == 0) {
+                const double al = d[1], w2 = d[0], v2 = d[2];
                 alpha[it] = al;
                 if (fabs(al) + bprev > scale) scale = fabs(al) + bprev;
                 const double b2 = w2 - 2.0 * al * al + al * al * v2;
@@ -1183,11 +1228,13 @@ __device__ void quad_lanczos_node(const QuadArgs& a, unsigned char* smem, uint32
                 tm_st8(k.tm + cb + z * 8, w);
             }
             tm_wait_st();
-            quad_warp_sum(acc, red[0]);
+            const float v1[1] = {acc};
+            quad_warp_sums<1>(v1, red);
             __syncthreads();
             if (warp == 0) {
-                const double b2 = quad_cta_sum(red[0]);
-                if (lane == 0) step_end(sqrt(b2));
+                double d[1];
+                quad_cta_sums<1>(red, d);
+                if (lane == 0) step_end(sqrt(d[0]));
             }
             __syncthreads();
         }
