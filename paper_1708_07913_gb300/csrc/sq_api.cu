@@ -279,7 +279,7 @@ int cluster_launch(sq_ctx* c, int which, const RegionArgs<float>& a, int blocks)
 // Allocates their per-CTA scratch and sets c->quad.
 int select_quad_kernels(sq_ctx* c)
 {
-    c->quad = 0;
+    c->quad[0] = c->quad[1] = 0;
     if (c->precision != SQ_FP32 || c->cl_nc > 0) return SQ_OK;
     const char* env = getenv("SQ_REGION_KERNEL");
     if (env && strcmp(env, "cta") == 0) return SQ_OK;
@@ -297,7 +297,8 @@ int select_quad_kernels(sq_ctx* c)
         if ((rc = dev_alloc(&c->d_qmask, sizeof(uint32_t) * c->lb * c->lb * (size_t)c->n_atoms))) return rc;
         if ((rc = launch_support_masks(c))) return rc;
     }
-    c->quad = 1;
+    c->quad[0] = 1;
+    c->quad[1] = !has_nl || c->g.m >= QD_MIN_NL_LANCZOS;
     return SQ_OK;
 }
 
@@ -340,7 +341,7 @@ int region_blocks(sq_ctx* c, int which, int* blocks)
         *blocks = (int)b;
         return SQ_OK;
     }
-    if (c->quad) {
+    if (c->quad[which]) {
         *blocks = (int)std::min<long long>(c->sm_count, c->g.Nd);
         return SQ_OK;
     }
@@ -383,7 +384,7 @@ int enqueue_bounds(sq_ctx* c, int blocks, int n_lanczos, double margin, double* 
         RegionArgs<float> a = region_args<float>(c);
         a.n_lanczos = n_lanczos; a.nl_cap = c->nl_cap; a.alpha = c->d_alpha; a.beta = c->d_beta; a.klen = c->d_klen;
         rc = c->cl_nc > 0 ? cluster_launch(c, 1, a, blocks)
-             : c->quad    ? launch_quad(c, 1, a, blocks)
+             : c->quad[1] ? launch_quad(c, 1, a, blocks)
                           : region_launch_f32(c->g.m, 1, a, region_extra(c, 1), blocks, c->stream);
     } else {
         RegionArgs<double> a = region_args<double>(c);
@@ -403,7 +404,7 @@ int enqueue_moments(sq_ctx* c, int blocks, const double* chi, const double* zeta
         RegionArgs<float> a = region_args<float>(c);
         a.chi = chi; a.zeta = zeta; a.moments = moments;
         rc = c->cl_nc > 0 ? cluster_launch(c, 0, a, blocks)
-             : c->quad    ? launch_quad(c, 0, a, blocks)
+             : c->quad[0] ? launch_quad(c, 0, a, blocks)
                           : region_launch_f32(c->g.m, 0, a, region_extra(c, 0), blocks, c->stream);
     } else {
         RegionArgs<double> a = region_args<double>(c);
@@ -444,7 +445,8 @@ struct sq_batch {
     int wait_unset = 0;
     // queue plan: groups of systems with one region half-width and precision
     struct Group {
-        int m = 0, prec = SQ_FP32, quad = 0;     // quad: its contexts run the quad kernels
+        int m = 0, prec = SQ_FP32;
+        int quad[2] = {0, 0};                    // its contexts run the quad kernels (moments, Lanczos)
         std::vector<int> sys;                    // batch indices, at most QMAX
         int bl = 0, bm = 0;                      // grids of the Lanczos and moments queue kernels
         size_t xl = 0, xm = 0;                   // their dynamic shared memory beyond the region vectors
@@ -599,42 +601,35 @@ int batch_build_queue(sq_batch* b, int npi)
         const sq_ctx* c = b->ctx[i];
         sq_batch::Group* g = nullptr;
         for (auto& x : G)
-            if (x.m == c->g.m && x.prec == c->precision && x.quad == c->quad && (int)x.sys.size() < QMAX) g = &x;
+            if (x.m == c->g.m && x.prec == c->precision && x.quad[0] == c->quad[0] && x.quad[1] == c->quad[1] && (int)x.sys.size() < QMAX) g = &x;
         if (!g) {
             G.emplace_back();
             g = &G.back();
             g->m = c->g.m;
             g->prec = c->precision;
-            g->quad = c->quad;
+            g->quad[0] = c->quad[0];
+            g->quad[1] = c->quad[1];
         }
         g->sys.push_back(i);
     }
     std::vector<QItem> items;
     for (auto& g : G) {
-        for (int i : g.sys) {
-            if (g.quad) {                        // xl, xm: all of the dynamic shared memory
-                g.xl = std::max(g.xl, b->ctx[i]->q_smem[1]);
-                g.xm = std::max(g.xm, b->ctx[i]->q_smem[0]);
-                continue;
-            }
-            g.xl = std::max(g.xl, region_extra(b->ctx[i], 1));
-            g.xm = std::max(g.xm, region_extra(b->ctx[i], 0));
-        }
         int bpl = 0, bpm = 0;
-        size_t sm = 0;
-        int rc;
-        if (g.quad) {
-            if ((rc = quad_queue_config(g.m, 1, g.xl)) || (rc = quad_queue_config(g.m, 0, g.xm))) return rc;
-            bpl = bpm = 1;
-        } else if ((rc = queue_config(g.prec, g.m, 1, g.xl, &bpl, &sm)) ||
-                   (rc = queue_config(g.prec, g.m, 0, g.xm, &bpm, &sm))) {
-            return rc;
+        for (int which = 1; which >= 0; --which) {
+            size_t& x = which ? g.xl : g.xm;     // quad: all of the dynamic shared memory, else beyond the region vectors
+            for (int i : g.sys) x = std::max(x, g.quad[which] ? b->ctx[i]->q_smem[which] : region_extra(b->ctx[i], which));
+            int& bps = which ? bpl : bpm;
+            size_t sm = 0;
+            bps = 1;
+            const int rc = g.quad[which] ? quad_queue_config(g.m, which, x) : queue_config(g.prec, g.m, which, x, &bps, &sm);
+            if (rc) return rc;
         }
+        int rc;
         const int sms = b->ctx[g.sys[0]]->sm_count;
         g.bl = bpl * sms;
         g.bm = bpm * sms;
         for (int i : g.sys)
-            if (!g.quad && (rc = ensure_scratch(b->ctx[i], std::max(g.bl, g.bm)))) return rc;
+            if ((rc = ensure_scratch(b->ctx[i], std::max(g.quad[1] ? 0 : g.bl, g.quad[0] ? 0 : g.bm)))) return rc;
         const int ns = (int)g.sys.size();
         g.need.assign(ns, 0);
         g.off_l = (int)items.size();
@@ -699,7 +694,7 @@ int queue_launch(const sq_batch* b, const sq_batch::Group& g, int which, const Q
 }
 int queue_launch(const sq_batch* b, const sq_batch::Group& g, int which, const QueueArgs<float>& q)
 {
-    if (!g.quad) return queue_launch(g.m, which, q, which ? g.xl : g.xm, which ? g.bl : g.bm, b->own);
+    if (!g.quad[which]) return queue_launch(g.m, which, q, which ? g.xl : g.xm, which ? g.bl : g.bm, b->own);
     QuadQueueArgs d;
     memset(&d, 0, sizeof(d));
     for (int k = 0; k < (int)g.sys.size(); ++k) {

@@ -157,10 +157,10 @@ struct sq_ctx {
     int cl_nc;
     int cl_clusters[2];
     size_t cl_smem[2];
-    // FP32 quad region kernels (sq_quad.cuh), one CTA per SM: in use (0: the
-    // general single-CTA kernels), their dynamic shared memory per kernel (0
-    // moments, 1 Lanczos) and per-CTA scratch
-    int quad;
+    // FP32 quad region kernels (sq_quad.cuh), one CTA per SM: in use, per kernel
+    // (0 moments, 1 Lanczos; else the general single-CTA kernel), their dynamic
+    // shared memory and per-CTA scratch
+    int quad[2];
     size_t q_smem[2];
     void* d_qscratch;
     uint32_t* d_qmask;               // support rows as column masks (QuadArgs::mask)

@@ -38,13 +38,19 @@
 namespace sq {
 
 constexpr int QD_MMAX = 15;                  // region half-widths 7 .. 15 have a quad kernel
-// From these half-widths on a context takes it.  One node per SM and a thread
-// per (quad, row pair) leave lanes and issue slots idle in small regions, of
-// which the general kernels keep several per SM: moments, general against quad
+// From these half-widths on a context takes it.  Speed: one node per SM and a
+// thread per (quad, row pair) leave lanes and issue slots idle in small regions,
+// of which the general kernels keep several per SM; moments, general against quad
 // kernel, cycles of one SM per node and step: with projectors 20.3K / 20.7K at
 // 13^3, 45.1K / 29.6K at 17^3, 127K / 64K at 29^3; local 7.2K / 9.2K at 13^3,
 // 14.6K / 11.8K at 17^3, 37.3K / 18.4K at 29^3.
-constexpr int QD_MIN_NL = 7, QD_MIN_LOCAL = 8;
+// Lanczos with projectors besides: in small regions extreme Ritz values that 40
+// FP32 steps leave unconverged move with the rounding, and the moments with them
+// (largest change over the moments' rms between the two kernels, seven seeded
+// systems each: 1e-2 at 17^3, 2e-3 at 19^3, 5e-4 at 21^3, 8e-5 at 23^3, 2e-5 at
+// 29^3; 5e-6 at most without projectors).  Those keep the general kernel's
+// rounding, whose own run-to-run spread is ten times smaller.
+constexpr int QD_MIN_NL = 7, QD_MIN_LOCAL = 8, QD_MIN_NL_LANCZOS = 11;
 constexpr int QD_NT = 512, QD_NW = 16;
 constexpr int QD_KMAX = 4 * ENTRIES_PER_ROW;  // list length per (quad, row pair, plane pair): four full rows
 constexpr int QD_ZERO = 504;                  // 8 TMEM columns of zeros: the planes beyond the region
