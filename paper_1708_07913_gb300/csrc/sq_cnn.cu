@@ -89,8 +89,6 @@ void free_bufs(sq_cnn* n)
 
 constexpr int LOSS_BLOCKS = 1024;
 
-long long nchunks(long long N) { return (N + CNN_CHUNK - 1) / CNN_CHUNK; }
-
 int ensure(sq_cnn* n, long long N)
 {
     if (N <= n->cap) return SQ_OK;
@@ -98,8 +96,7 @@ int ensure(sq_cnn* n, long long N)
     free_bufs(n);
     const size_t ts = n->bf16 ? sizeof(Bf16) : sizeof(float);
     const size_t NC = (size_t)N * C;
-    const size_t part = (size_t)nchunks(N) * std::max({(size_t)(T1 + 1) * C, (size_t)(T2 + 1) * C * C,
-                                                       (size_t)(T3 + 1) * C});
+    const size_t part = (size_t)CNN_PARTS * std::max({(size_t)(T1 + 1) * C, (size_t)(T2 + 1) * C * C, (size_t)(T3 + 1) * C});
     int rc;
     if ((rc = alloc(&n->x0, ts * N)) || (rc = alloc(&n->a1, ts * NC)) || (rc = alloc(&n->a2, ts * NC)) ||
         (rc = alloc(&n->z1, 4 * NC)) || (rc = alloc(&n->z2, 4 * NC)) || (rc = alloc(&n->y, 4 * (size_t)N)) ||
@@ -118,36 +115,46 @@ int grid_for(long long work, int sm)
     return (int)std::max<long long>(1, std::min<long long>(b, (long long)sm * 16));
 }
 
+// Dynamic shared memory beyond the 48 KB default (the limit only ever grows).
+int smem_limit(const void* fn, size_t bytes)
+{
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) return SQ_ECUDA;
+    if ((int)bytes > fa.maxDynamicSharedSizeBytes &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+        return SQ_ECUDA;
+    return SQ_OK;
+}
+
+int tile_grid(long long tiles, long long most) { return (int)std::max<long long>(1, std::min(tiles, most)); }
+
+// keep: also store what the backward pass reads (pre-activations and y).
 template <typename T>
-int forward_t(sq_cnn* n, const CnnGrid& g, const double* V, double* rho)
+int forward_t(sq_cnn* n, const CnnGrid& g, const double* V, double* rho, bool keep)
 {
     const T* wt = (const T*)n->wt;
     T* x0 = (T*)n->x0;
     T* a1 = (T*)n->a1;
     T* a2 = (T*)n->a2;
-    const int gN = grid_for(g.N, n->sm), gNC = grid_for(g.N * C, n->sm);
-    cnn_input_kernel<T><<<gN, CNN_NT, 0, n->st>>>(g, V, n->v_shift + n->shift, n->v_scale, x0);
-    cnn_conv_fwd_kernel<T, 1, 5><<<gNC, CNN_NT, 0, n->st>>>(g, x0, wt + OW1, n->w + OB1, n->z1, a1);
-    if constexpr (sizeof(T) == sizeof(Bf16)) {
-        if (n->tensor) {
-            static bool attr = false;        // the kernel's shared memory exceeds the 48 KB default
-            if (!attr) {
-                if (cudaFuncSetAttribute(cnn_conv2_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM) !=
-                    cudaSuccess)
-                    return SQ_ECUDA;
-                attr = true;
-            }
-            const long long tiles = (g.N + TC_M - 1) / TC_M;
-            const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, (long long)n->sm));
-            cnn_conv2_tc_kernel<<<grid, 128, TC_SMEM, n->st>>>(g, (const Bf16*)a1, (const Bf16*)(wt + OW2),
-                                                               n->w + OB2, n->z2, (Bf16*)a2, n->err);
-        } else {
-            cnn_conv_fwd_kernel<T, C, 3><<<gNC, CNN_NT, 0, n->st>>>(g, a1, wt + OW2, n->w + OB2, n->z2, a2);
-        }
+    float *z1 = keep ? n->z1 : nullptr, *z2 = keep ? n->z2 : nullptr;
+    int rc;
+    cnn_input_kernel<T><<<grid_for(g.N, n->sm), CNN_NT, 0, n->st>>>(g, V, n->v_shift + n->shift, n->v_scale, x0);
+    cnn_conv1_kernel<T><<<tile_grid(cnn_tiles<C1_X, C1_Y, C1_Z>(g), (long long)n->sm * 4), CNN_NT, 0, n->st>>>(
+        g, x0, wt + OW1, n->w + OB1, z1, a1);
+    bool tensor = false;
+    if constexpr (sizeof(T) == sizeof(Bf16)) tensor = n->tensor;
+    if (tensor) {
+        if ((rc = smem_limit((const void*)cnn_conv2_tc_kernel, TC_SMEM))) return rc;
+        cnn_conv2_tc_kernel<<<tile_grid(cnn_tiles<TC_X, TC_Y, 1>(g), (long long)n->sm * 2), TC_T, TC_SMEM, n->st>>>(
+            g, (const Bf16*)a1, (const Bf16*)(wt + OW2), n->w + OB2, z2, (Bf16*)a2, n->err);
     } else {
-        cnn_conv_fwd_kernel<T, C, 3><<<gNC, CNN_NT, 0, n->st>>>(g, a1, wt + OW2, n->w + OB2, n->z2, a2);
+        if ((rc = smem_limit((const void*)cnn_conv2_kernel<T, T, false>, C2_SMEM))) return rc;
+        cnn_conv2_kernel<T, T, false><<<tile_grid(cnn_tiles<C2_X, C2_Y, C2_Z>(g), (long long)n->sm * 3), C2_T, C2_SMEM, n->st>>>(
+            g, a1, wt + OW2, n->w + OB2, nullptr, z2, a2);
     }
-    cnn_out_fwd_kernel<T><<<gN, CNN_NT, 0, n->st>>>(g, a2, wt + OW3, n->w + OB3, n->rho_scale, n->y, rho);
+    if ((rc = smem_limit((const void*)cnn_out_fwd_kernel<T>, c3_smem<T>()))) return rc;
+    cnn_out_fwd_kernel<T><<<tile_grid(cnn_tiles<C3_X, C3_Y, C3_Z>(g), (long long)n->sm * 4), CNN_NT, c3_smem<T>(), n->st>>>(
+        g, a2, wt + OW3, n->w + OB3, n->rho_scale, keep ? n->y : nullptr, rho);
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
 
@@ -166,23 +173,30 @@ template <typename T>
 int backward_t(sq_cnn* n, const CnnGrid& g, const double* ref, const double* rho, int accumulate)
 {
     const T* wt = (const T*)n->wt;
-    const int gN = std::min(grid_for(g.N, n->sm), LOSS_BLOCKS), gNC = grid_for(g.N * C, n->sm);
+    const int gN = std::min(grid_for(g.N, n->sm), LOSS_BLOCKS);
+    const int nc = tile_grid(cnn_tiles<WG_X, WG_Y, WG_Z>(g), CNN_PARTS);
+    int rc;
+    if ((rc = smem_limit((const void*)cnn_wgrad3_kernel<T>, WG3_SMEM)) ||
+        (rc = smem_limit((const void*)cnn_wgrad2_kernel<T>, WG2_SMEM)) ||
+        (rc = smem_limit((const void*)cnn_conv2_kernel<float, T, true>, C2_SMEM)))
+        return rc;
     cnn_loss_kernel<<<gN, CNN_NT, 0, n->st>>>(g, rho, ref, n->y, n->rho_scale, n->gy, n->lpart);
     cnn_loss_sum_kernel<<<1, 32, 0, n->st>>>(n->lpart, gN, 1.0 / ((double)g.N * n->rho_scale * n->rho_scale),
                                              n->lout);
-    const int nc = (int)nchunks(g.N);
     // output layer: weights, then the data gradient into the second layer
-    cnn_wgrad_kernel<T, C, 1, 3><<<dim3(nc, T3 + 1), CNN_NT, 0, n->st>>>(g, n->gy, (const T*)n->a2, n->part);
+    cnn_wgrad3_kernel<T><<<nc, CNN_NT, WG3_SMEM, n->st>>>(g, n->gy, (const T*)n->a2, n->part);
     cnn_wgrad_sum_kernel<<<grid_for((long long)(T3 + 1) * C, n->sm), CNN_NT, 0, n->st>>>(
         n->part, nc, T3 + 1, C, 1, n->g + OW3, n->g + OB3, accumulate);
-    cnn_conv_bwd_data_kernel<T, 1, 3><<<gNC, CNN_NT, 0, n->st>>>(g, n->gy, wt + OW3, n->z2, n->gz2);
+    cnn_out_bwd_kernel<T><<<tile_grid(cnn_tiles<8, 8, 2>(g), (long long)n->sm * 8), CNN_NT, 0, n->st>>>(
+        g, n->gy, wt + OW3, n->z2, n->gz2);
     // second layer
-    cnn_wgrad_kernel<T, C, C, 3><<<dim3(nc, T2 + 1), CNN_NT, 0, n->st>>>(g, n->gz2, (const T*)n->a1, n->part);
+    cnn_wgrad2_kernel<T><<<dim3(nc, 3), CNN_NT, WG2_SMEM, n->st>>>(g, n->gz2, (const T*)n->a1, n->part);
     cnn_wgrad_sum_kernel<<<grid_for((long long)(T2 + 1) * C * C, n->sm), CNN_NT, 0, n->st>>>(
         n->part, nc, T2 + 1, C * C, C, n->g + OW2, n->g + OB2, accumulate);
-    cnn_conv_bwd_data_kernel<T, C, 3><<<gNC, CNN_NT, 0, n->st>>>(g, n->gz2, wt + OW2, n->z1, n->gz1);
+    cnn_conv2_kernel<float, T, true><<<tile_grid(cnn_tiles<C2_X, C2_Y, C2_Z>(g), (long long)n->sm * 3), C2_T, C2_SMEM, n->st>>>(
+        g, n->gz2, wt + OW2, nullptr, n->z1, n->gz1, (T*)nullptr);
     // first layer
-    cnn_wgrad_kernel<T, 1, C, 5><<<dim3(nc, T1 + 1), CNN_NT, 0, n->st>>>(g, n->gz1, (const T*)n->x0, n->part);
+    cnn_wgrad1_kernel<T><<<nc, CNN_NT, 0, n->st>>>(g, n->gz1, (const T*)n->x0, n->part);
     cnn_wgrad_sum_kernel<<<grid_for((long long)(T1 + 1) * C, n->sm), CNN_NT, 0, n->st>>>(
         n->part, nc, T1 + 1, C, C, n->g + OW1, n->g + OB1, accumulate);
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
@@ -343,7 +357,7 @@ int sq_cnn_forward(sq_cnn* n, int n1, int n2, int n3, const double* V, double* r
     CnnGrid g{n1, n2, n3, (long long)n1 * n2 * n3};
     int rc = ensure(n, g.N);
     if (rc) return rc;
-    return n->bf16 ? forward_t<Bf16>(n, g, V, rho) : forward_t<float>(n, g, V, rho);
+    return n->bf16 ? forward_t<Bf16>(n, g, V, rho, false) : forward_t<float>(n, g, V, rho, false);
 }
 
 int sq_cnn_set_shift(sq_cnn* n, double shift)
@@ -378,7 +392,7 @@ int sq_cnn_backward(sq_cnn* n, int n1, int n2, int n3, const double* V, const do
     CnnGrid g{n1, n2, n3, (long long)n1 * n2 * n3};
     int rc = ensure(n, g.N);
     if (rc) return rc;
-    rc = n->bf16 ? forward_t<Bf16>(n, g, V, rho) : forward_t<float>(n, g, V, rho);
+    rc = n->bf16 ? forward_t<Bf16>(n, g, V, rho, true) : forward_t<float>(n, g, V, rho, true);
     if (rc) return rc;
     rc = n->bf16 ? backward_t<Bf16>(n, g, rho_ref, rho, accumulate) : backward_t<float>(n, g, rho_ref, rho, accumulate);
     if (rc) return rc;
