@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(CNN_NT) cnn_out_bwd_kernel(CnnGrid g, const fl
 // its neighbours and G in shared memory (zero beyond the grid); rows of 8 nodes
 // along x share the loads of A between the taps dx and those of G between dy.
 // 16^3 nodes: a block per (4096 nodes, tap), each node in turn, took 464 us for the
-// middle layer, 374 for the last and 898 for the first; these take 21, 20 and under 13.
+// middle layer, 374 for the last and 898 for the first; these take 21, 20 and 11.
 constexpr int WG_X = 8, WG_Y = 8, WG_Z = 2;
 
 // Middle layer (32 x 32 per tap): slab = dz, a thread has one input, four outputs and the slab's 9 taps.

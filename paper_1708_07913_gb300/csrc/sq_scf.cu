@@ -27,6 +27,39 @@ constexpr int T_RED = 256;          // threads per reduction block
 constexpr int MAX_RED_BLOCKS = 1024;
 constexpr int MAX_HIST = 16;        // Anderson history
 
+// Sum of one value per thread over the grid: a tree per block, the block
+// partials by the last block, in a fixed order.  True in thread 0 of the last
+// block, which then has the total in s.
+__device__ inline bool grid_total(double& s, double* partials, unsigned* counter)
+{
+    __shared__ double sh[T_RED / 32];
+    __shared__ bool last;
+    auto block_total = [&]() {
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s = 0.0;
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
+        }
+    };
+    block_total();
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    s = 0.0;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) s += __ldcg(partials + b);
+    __syncthreads();
+    block_total();
+    if (threadIdx.x == 0) *counter = 0;
+    return threadIdx.x == 0;
+}
+
 // sum over t of A(t) B(t), A = a1 - a0, B = b1 - b0 (a0, b0 may be NULL;
 // b1 NULL means B = 1).  Block partials, then the last block adds them in
 // index order into *out and resets the counter.
@@ -34,32 +67,13 @@ __global__ void dot_kernel(const double* __restrict__ a1, const double* __restri
                            const double* __restrict__ b1, const double* __restrict__ b0, long long n,
                            double* partials, unsigned* counter, double* out)
 {
-    __shared__ double sh[T_RED / 32];
-    __shared__ bool last;
     double s = 0.0;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
         const double A = a0 ? a1[t] - a0[t] : a1[t];
         const double B = b1 ? (b0 ? b1[t] - b0[t] : b1[t]) : 1.0;
         s += A * B;
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double b = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b += sh[w];
-        partials[blockIdx.x] = b;
-        __threadfence();
-        last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last && threadIdx.x == 0) {
-        __threadfence();
-        double tot = 0.0;
-        for (unsigned b = 0; b < gridDim.x; ++b) tot += ((volatile double*)partials)[b];
-        *out = tot;
-        *counter = 0;
-    }
+    if (grid_total(s, partials, counter)) *out = s;
 }
 
 // max over t of |a(t) - b(t)|, block maxima then the last block's maximum in
@@ -104,30 +118,101 @@ __global__ void widen_kernel(const double* __restrict__ chi_ref, const double* _
     }
 }
 
-// y = -lap_h x on the periodic grid (x fastest): the d = 0 term of
-// Eq. (FD:Laplacian) appears in its six axis terms.
 struct FDW {
     double w[FD_NO + 1];
 };
-__global__ void lap_periodic_kernel(const double* __restrict__ x, double* __restrict__ y, int n1, int n2, int n3,
-                                    FDW fw)
+
+// ------------------------------------------------------------------------
+// Conjugate gradients for (-lap_h + shift) u = f on the periodic grid, x
+// fastest (the d = 0 term of Eq. (FD:Laplacian) appears in its six axis terms).
+// The scalars stay on the device: every kernel's last block turns its sum into
+// the step length or the direction's factor and decides whether the iteration
+// ends; the kernels of the iterations past the end return at once, so the host
+// only looks every CG_LOT iterations.  Three launches per iteration, none of
+// them waited for: at 64^3 an iteration took 146 us with five launches and two
+// host waits, 46 us now (31 + 11 + 4), of which the operator's 43 FP64 operations per point
+// (two lanes per clock and SM) are 18 us.
+// ------------------------------------------------------------------------
+enum { CG_RR = 0, CG_ALPHA, CG_BETA, CG_LIMIT, CG_DONE, CG_ITERS, CG_MAX, CG_NSTATE };
+constexpr int CG_LOT = 32;
+
+// Start: rr = |f|^2 (given), the limit on |r| and on the iterations.
+__global__ void cg_start_kernel(double* st, double rr, double limit, int max_iter)
 {
+    st[CG_RR] = rr;
+    st[CG_ALPHA] = st[CG_BETA] = st[CG_ITERS] = 0.0;
+    st[CG_LIMIT] = limit;
+    st[CG_MAX] = (double)max_iter;
+    st[CG_DONE] = !(sqrt(rr) > limit) || max_iter < 1 ? 1.0 : 0.0;
+}
+
+// i + d on an axis of n points, |d| <= FD_NO
+__device__ inline int cg_wrap(int i, int n)
+{
+    if (n >= FD_NO) return i < 0 ? i + n : i >= n ? i - n : i;
+    const int r = i % n;
+    return r < 0 ? r + n : r;
+}
+
+// Ap = (-lap_h + shift) p, then alpha = rr / (p . Ap).
+__global__ void __launch_bounds__(T_RED) cg_apply_kernel(const double* __restrict__ p, double* __restrict__ Ap, int n1,
+                                                         int n2, int n3, FDW fw, double shift, double* partials,
+                                                         unsigned* counter, double* st)
+{
+    if (st[CG_DONE] != 0.0) return;                       // uniform over the grid
     const long long n = (long long)n1 * n2 * n3;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(p % n1), j = (int)((p / n1) % n2), k = (int)(p / ((long long)n1 * n2));
-        const long long row = p - i, plane = p - i - (long long)j * n1;
-        double acc = 6.0 * fw.w[0] * x[p];
+    double s = 0.0;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
+        const int i = (int)(t % n1), j = (int)((t / n1) % n2), k = (int)(t / ((long long)n1 * n2));
+        const double* row = p + (t - i);
+        const double* col = p + ((long long)k * n2 * n1 + i);
+        const double* pil = p + ((long long)j * n1 + i);
+        const long long pl = (long long)n1 * n2;
+        const double x = p[t];
+        double acc = 6.0 * fw.w[0] * x;
+#pragma unroll
         for (int d = 1; d <= FD_NO; ++d) {
-            const int ip = (i + d) % n1, im = ((i - d) % n1 + n1) % n1;
-            const int jp = (j + d) % n2, jm = ((j - d) % n2 + n2) % n2;
-            const int kp = (k + d) % n3, km = ((k - d) % n3 + n3) % n3;
-            const double sx = x[row + ip] + x[row + im];
-            const double sy = x[plane + (long long)jp * n1 + i] + x[plane + (long long)jm * n1 + i];
-            const double sz = x[((long long)kp * n2 + j) * n1 + i] + x[((long long)km * n2 + j) * n1 + i];
+            const double sx = row[cg_wrap(i + d, n1)] + row[cg_wrap(i - d, n1)];
+            const double sy = col[(long long)cg_wrap(j + d, n2) * n1] + col[(long long)cg_wrap(j - d, n2) * n1];
+            const double sz = pil[cg_wrap(k + d, n3) * pl] + pil[cg_wrap(k - d, n3) * pl];
             acc += fw.w[d] * ((sx + sy) + sz);
         }
-        y[p] = -acc;
+        const double y = shift * x - acc;
+        Ap[t] = y;
+        s += x * y;
     }
+    if (grid_total(s, partials, counter)) st[CG_ALPHA] = st[CG_RR] / s;
+}
+
+// u += alpha p, r -= alpha Ap, then beta = rr' / rr, and the end of the iteration.
+__global__ void __launch_bounds__(T_RED) cg_step_kernel(double* __restrict__ u, double* __restrict__ r,
+                                                        const double* __restrict__ p, const double* __restrict__ Ap,
+                                                        long long n, double* partials, unsigned* counter, double* st)
+{
+    if (st[CG_DONE] != 0.0) return;
+    const double alpha = st[CG_ALPHA];
+    double s = 0.0;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
+        u[t] += alpha * p[t];
+        const double v = r[t] - alpha * Ap[t];
+        r[t] = v;
+        s += v * v;
+    }
+    if (!grid_total(s, partials, counter)) return;
+    st[CG_BETA] = s / st[CG_RR];
+    st[CG_RR] = s;
+    st[CG_ITERS] += 1.0;
+    if (!(sqrt(s) > st[CG_LIMIT]) || st[CG_ITERS] >= st[CG_MAX]) st[CG_DONE] = 1.0;
+}
+
+// p = r + beta p
+__global__ void __launch_bounds__(T_RED) cg_direction_kernel(double* __restrict__ p, const double* __restrict__ r,
+                                                             long long n, const double* st)
+{
+    if (st[CG_DONE] != 0.0) return;
+    const double beta = st[CG_BETA];
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
+        p[t] = r[t] + beta * p[t];
 }
 
 __global__ void rhs_kernel(const double* __restrict__ rho, const double* mean, double* __restrict__ b, long long n)
@@ -142,21 +227,6 @@ __global__ void shift_kernel(double* __restrict__ x, const double* sum, long lon
     const double m = *sum / (double)n;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
         x[t] -= m;
-}
-
-__global__ void cg_update_kernel(double* __restrict__ phi, double* __restrict__ r, const double* __restrict__ p,
-                                 const double* __restrict__ Ap, double alpha, long long n)
-{
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-        phi[t] += alpha * p[t];
-        r[t] -= alpha * Ap[t];
-    }
-}
-
-__global__ void xpby_kernel(double* __restrict__ p, const double* __restrict__ r, double beta, long long n)
-{
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
-        p[t] = r[t] + beta * p[t];
 }
 
 // V_out = V_loc + phi + v_x(rho), v_x = -(3 alpha / 2) (3 rho / pi)^(1/3) (0 for rho <= 0)
@@ -193,28 +263,6 @@ __global__ void sub_kernel(const double* __restrict__ a, const double* __restric
 {
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
         out[t] = a[t] - b[t];
-}
-
-// y = -lap_h x + s x on the periodic grid (the operator of the preconditioner)
-__global__ void helmholtz_kernel(const double* __restrict__ x, double* __restrict__ y, int n1, int n2, int n3,
-                                 FDW fw, double s)
-{
-    const long long n = (long long)n1 * n2 * n3;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(p % n1), j = (int)((p / n1) % n2), k = (int)(p / ((long long)n1 * n2));
-        const long long row = p - i, plane = p - i - (long long)j * n1;
-        double acc = 6.0 * fw.w[0] * x[p];
-        for (int d = 1; d <= FD_NO; ++d) {
-            const int ip = (i + d) % n1, im = ((i - d) % n1 + n1) % n1;
-            const int jp = (j + d) % n2, jm = ((j - d) % n2 + n2) % n2;
-            const int kp = (k + d) % n3, km = ((k - d) % n3 + n3) % n3;
-            const double sx = x[row + ip] + x[row + im];
-            const double sy = x[plane + (long long)jp * n1 + i] + x[plane + (long long)jm * n1 + i];
-            const double sz = x[((long long)kp * n2 + j) * n1 + i] + x[((long long)km * n2 + j) * n1 + i];
-            acc += fw.w[d] * ((sx + sy) + sz);
-        }
-        y[p] = s * x[p] - acc;
-    }
 }
 
 // out = v_in + f - c u (u is read from out)
@@ -277,6 +325,43 @@ int read_slots(Red& R, double* host, int count, cudaStream_t st)
     return SQ_OK;
 }
 
+// Run the conjugate gradients for (-lap_h + shift) u = f from u = 0, r = p = f
+// (u, r, p set by the caller, rr = |f|^2) until |r| <= limit or max_iter
+// iterations; the scalars live in R.out[CG_AT..].
+constexpr int CG_AT = 8;
+int run_cg(sq_ctx* c, Red& R, double* u, double* r, double* p, double* Ap, const FDW& fw, double shift, double rr0,
+           double limit, int max_iter, int* iters, double* rr_end)
+{
+    const long long n = c->g.Nd;
+    cudaStream_t st = c->stream;
+    const int G = (int)std::max<long long>(1, std::min<long long>((n + T_RED - 1) / T_RED, R.blocks));
+    double* S = R.out + CG_AT;
+    cg_start_kernel<<<1, 1, 0, st>>>(S, rr0, limit, max_iter);
+    c->launches++;
+    *iters = 0;
+    *rr_end = rr0;
+    if (!(sqrt(rr0) > limit) || max_iter < 1) return SQ_OK;
+    double h[CG_NSTATE];
+    for (;;) {
+        for (int i = 0; i < CG_LOT; ++i) {
+            cg_apply_kernel<<<G, T_RED, 0, st>>>(p, Ap, c->g.n1, c->g.n2, c->g.n3, fw, shift, R.partials, R.counter, S);
+            cg_step_kernel<<<G, T_RED, 0, st>>>(u, r, p, Ap, n, R.partials, R.counter, S);
+            cg_direction_kernel<<<G, T_RED, 0, st>>>(p, r, n, S);
+        }
+        c->launches += 3 * CG_LOT;
+        if (cudaGetLastError() != cudaSuccess) return SQ_ECUDA;
+        if (cudaMemcpyAsync(h, S, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess) {
+            cudaGetLastError();
+            return SQ_ECUDA;
+        }
+        if (h[CG_DONE] != 0.0) break;
+    }
+    *iters = (int)h[CG_ITERS];
+    *rr_end = h[CG_RR];
+    return SQ_OK;
+}
+
 int read_slot(Red& R, int slot, double* host, cudaStream_t st)
 {
     if (cudaMemcpyAsync(host, R.out + slot, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -335,7 +420,7 @@ int context_ws(sq_ctx* c, PoissonWS** out)
         ws = new (std::nothrow) PoissonWS();
         if (!ws) return SQ_ENOMEM;
         int rc = cudaMalloc(&ws->buf, sizeof(double) * 4 * n) == cudaSuccess ? SQ_OK : SQ_ENOMEM;
-        if (rc == SQ_OK) rc = red_alloc(ws->red, c->sm_count, 8);
+        if (rc == SQ_OK) rc = red_alloc(ws->red, c->sm_count, CG_AT + CG_NSTATE);
         if (rc) {
             cudaGetLastError();
             ws_free(ws);
@@ -454,20 +539,7 @@ int sq_poisson(sq_ctx* c, const double* rho, double* phi, double tol, int max_it
         if (cudaMemcpyAsync(r, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
             cudaMemcpyAsync(p, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
             return SQ_ECUDA;
-        while (sqrt(rr) > tol * bnorm && it < max_iter) {
-            lap_periodic_kernel<<<G, 256, 0, st>>>(p, Ap, c->g.n1, c->g.n2, c->g.n3, fw);
-            if ((rc = enqueue_dot(R, p, nullptr, Ap, nullptr, n, 4, st))) return rc;
-            double pAp, rr_new;
-            if ((rc = read_slot(R, 4, &pAp, st))) return rc;
-            const double alpha = rr / pAp;
-            cg_update_kernel<<<G, 256, 0, st>>>(phi, r, p, Ap, alpha, n);
-            if ((rc = enqueue_dot(R, r, nullptr, r, nullptr, n, 5, st))) return rc;
-            if ((rc = read_slot(R, 5, &rr_new, st))) return rc;
-            xpby_kernel<<<G, 256, 0, st>>>(p, r, rr_new / rr, n);
-            c->launches += 5;
-            rr = rr_new;
-            ++it;
-        }
+        if ((rc = run_cg(c, R, phi, r, p, Ap, fw, 0.0, rr, tol * bnorm, max_iter, &it, &rr))) return rc;
         if ((rc = enqueue_dot(R, phi, nullptr, nullptr, nullptr, n, 6, st))) return rc;   // phi mean-free
         shift_kernel<<<G, 256, 0, st>>>(phi, R.out + 6, n);
         c->launches += 2;
@@ -548,20 +620,7 @@ int sq_kerker(sq_ctx* c, const double* v_in, const double* v_out, double k0, dou
         return SQ_ECUDA;
     double rr = h2[0];
     int it = 0;
-    while (fnorm > 0.0 && sqrt(rr) > tol * fnorm && it < max_iter) {
-        helmholtz_kernel<<<G, 256, 0, st>>>(p, Ap, c->g.n1, c->g.n2, c->g.n3, fw, s);
-        if ((rc = enqueue_dot(R, p, nullptr, Ap, nullptr, n, 4, st))) return rc;
-        double pAp, rr_new;
-        if ((rc = read_slot(R, 4, &pAp, st))) return rc;
-        const double alpha = rr / pAp;
-        cg_update_kernel<<<G, 256, 0, st>>>(u, r, p, Ap, alpha, n);
-        if ((rc = enqueue_dot(R, r, nullptr, r, nullptr, n, 5, st))) return rc;
-        if ((rc = read_slot(R, 5, &rr_new, st))) return rc;
-        xpby_kernel<<<G, 256, 0, st>>>(p, r, rr_new / rr, n);
-        c->launches += 5;
-        rr = rr_new;
-        ++it;
-    }
+    if (fnorm > 0.0 && (rc = run_cg(c, R, u, r, p, Ap, fw, s, rr, tol * fnorm, max_iter, &it, &rr))) return rc;
     kerker_out_kernel<<<G, 256, 0, st>>>(v_in, f, (1.0 - amin) * s, v_pre, n);
     c->launches++;
     if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess) return SQ_ECUDA;
