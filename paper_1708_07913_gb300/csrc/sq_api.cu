@@ -290,33 +290,18 @@ int select_quad_kernels(sq_ctx* c)
         if (rc == SQ_EUNSUPPORTED) return SQ_OK;
         if (rc) return rc;
     }
-    c->q_stride = quad_scratch(c->g.m, has_nl ? c->ccap : 0, has_nl ? c->lb : 0).total;
-    int rc = dev_alloc(&c->d_qscratch, c->q_stride * (size_t)c->sm_count);       // one CTA per SM, a queue's too
-    if (rc) return rc;
+    int rc;
     if (has_nl) {
-        if ((rc = dev_alloc(&c->d_qmask, sizeof(uint32_t) * c->lb * c->lb * (size_t)c->n_atoms))) return rc;
-        if ((rc = launch_support_masks(c))) return rc;
+        int most = 0;
+        if ((rc = dev_alloc(&c->d_qmask, sizeof(uint32_t) * (c->lb * c->lb * (size_t)c->n_atoms + 1)))) return rc;
+        if ((rc = launch_support_masks(c, &most))) return rc;
+        if (most > ENTRIES_PER_ROW) return SQ_OK;          // the general kernels refuse such rows
     }
+    c->q_stride = quad_scratch(c->g.m, has_nl ? c->ccap : 0, has_nl ? c->lb : 0).total;
+    if ((rc = dev_alloc(&c->d_qscratch, c->q_stride * (size_t)c->sm_count))) return rc;   // one CTA per SM, a queue's too
     c->quad[0] = 1;
     c->quad[1] = !has_nl || c->g.m >= QD_MIN_NL_LANCZOS;
     return SQ_OK;
-}
-
-// Arguments of the quad kernels with the region arguments a.
-QuadArgs quad_args(const sq_ctx* c, const RegionArgs<float>& a)
-{
-    QuadArgs q;
-    memset(&q, 0, sizeof(q));
-    q.r = a;
-    for (int d = 0; d <= FD_NO; ++d) q.wd2[d] = make_float2(a.wd[d], a.wd[d]);
-    q.diag = (float)(-3.0 * c->g.w[0]);
-    q.scratch = (char*)c->d_qscratch;
-    q.stride = c->q_stride;
-    q.mask = c->d_qmask;
-    q.nxq = quad_nxq(c->lb);
-    q.nyp = quad_nyp(c->lb);
-    q.recs = quad_recs(c->lb);
-    return q;
 }
 
 // Launch quad kernel `which` with the region arguments a.

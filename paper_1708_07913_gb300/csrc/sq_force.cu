@@ -1,7 +1,8 @@
 // sq_force.cu -- host side of sq_nl_forces (include/sq.h): argument checks,
 // the per-context force workspace, and the two launches: a per-node force
-// kernel (by default the region form of sq_force_region.cuh, which runs the
-// recurrence on the region kernels' machinery; the first form of
+// kernel (by default the quad form of sq_quad_force.cuh in contexts that run the
+// quad kernels, else the region form of sq_force_region.cuh, which runs the
+// recurrence on the general region kernels' machinery; the first form of
 // sq_force.cuh where the region form does not fit, or with
 // SQ_FORCE_KERNEL=legacy in the environment) and the fixed-order sum over
 // its CTAs.
@@ -17,6 +18,7 @@
 
 #include "sq_force.cuh"
 #include "sq_force_region.cuh"
+#include "sq_quad_force.cuh"
 
 using namespace sq;
 
@@ -26,6 +28,9 @@ int force_region_config_f32(int m, size_t extra, int* bps, size_t* smem);
 int force_region_config_f64(int m, size_t extra, int* bps, size_t* smem);
 int force_region_launch_f32(int m, const ForceRegionArgs<float>& f, size_t extra, int blocks, cudaStream_t st);
 int force_region_launch_f64(int m, const ForceRegionArgs<double>& f, size_t extra, int blocks, cudaStream_t st);
+int quad_force_config(int m, int ccap, int lb, int npl, size_t* smem);
+int quad_force_launch(int m, const QuadForceArgs& f, size_t smem, int blocks, cudaStream_t st);
+int launch_chebyshev_table(int npl, double* tab, cudaStream_t st);
 }
 
 // Per-context scratch of the force kernel (created on first use, grown when
@@ -251,6 +256,60 @@ int launch_force_region(sq_ctx* c, const RegionForceLayout& L, char* base, int b
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
 
+// Grid of the quad form (0: not available for this context).
+int quad_force_blocks(sq_ctx* c, long long nq, size_t* smem)
+{
+    const char* env = getenv("SQ_FORCE_KERNEL");
+    if (!c->quad[0] || (env && (strcmp(env, "legacy") == 0 || strcmp(env, "region") == 0))) return 0;
+    if (quad_force_config(c->g.m, c->ccap, c->lb, c->npl, smem)) return 0;
+    return (int)std::min<long long>(c->sm_count, nq);
+}
+
+// Workspace of the quad form: per CTA D, one node's contributions and the CTA's
+// force array, then the Chebyshev table.
+struct QuadForceLayout {
+    size_t D, fpart, F, cta, tab;
+};
+
+QuadForceLayout quad_force_layout(int S, int n_atoms, int npl)
+{
+    QuadForceLayout L;
+    L.D = 0;
+    L.fpart = align256((size_t)4 * S * 2 * 32 * 16);
+    L.F = L.fpart + align256(sizeof(double) * 3 * MAX_CAND);
+    L.cta = L.F + align256(sizeof(double) * 3 * (size_t)n_atoms);
+    L.tab = align256(sizeof(double) * (size_t)(npl + 1) * (npl + 1));
+    return L;
+}
+
+int launch_force_quad(sq_ctx* c, const QuadForceLayout& L, char* base, int blocks, size_t smem, const double* chi,
+                      const double* zeta, double mu, double kT, const long long* nodes, long long nq, double* forces)
+{
+    QuadForceArgs f;
+    memset(&f, 0, sizeof(f));
+    RegionArgs<float> r = region_args<float>(c);
+    r.chi = chi;
+    r.zeta = zeta;
+    f.q = quad_args(c, r);
+    grad_weights(FD_NO, c->g.h, f.grad);
+    f.mu = mu;
+    f.kT = kT;
+    f.nodes = nodes;
+    f.nq = nq;
+    f.D = (float4*)(base + L.D * blocks);
+    f.fpart = (double*)(base + L.fpart * blocks);
+    f.Fcta = (double*)(base + L.F * blocks);
+    double* tab = (double*)(base + L.cta * blocks);
+    f.ctab = tab;
+    int rc = launch_chebyshev_table(c->npl, tab, c->stream);
+    if (rc) return rc;
+    if ((rc = quad_force_launch(c->g.m, f, smem, blocks, c->stream))) return rc;
+    c->launches++;
+    const int n3 = 3 * c->n_atoms;
+    force_sum_kernel<<<(n3 + 127) / 128, 128, 0, c->stream>>>(f.Fcta, blocks, n3, forces);
+    return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
+}
+
 // The context's force workspace, at least `need` bytes.
 int force_workspace(sq_ctx* c, size_t need, ForceWS** out)
 {
@@ -327,8 +386,14 @@ int nl_forces(sq_ctx* c, const double* V, const double* chi, const double* zeta,
     ForceWS* ws = nullptr;
     int rc;
     size_t extra = 0;
-    const int rblocks = region_force_blocks(c, nq, &extra);
-    if (rblocks > 0) {
+    const int qblocks = quad_force_blocks(c, nq, &extra);
+    const int rblocks = qblocks > 0 ? 0 : region_force_blocks(c, nq, &extra);
+    if (qblocks > 0) {
+        const QuadForceLayout L = quad_force_layout(S, c->n_atoms, c->npl);
+        if ((rc = force_workspace(c, L.cta * (size_t)qblocks + L.tab, &ws))) return rc;
+        if ((rc = launch_build_vpad(c, V))) return rc;
+        rc = launch_force_quad(c, L, ws->buf, qblocks, extra, chi, zeta, mu, kT, nodes, nq, forces);
+    } else if (rblocks > 0) {
         const RegionForceLayout L = region_force_layout(S, c->n_atoms, tsz);
         if ((rc = force_workspace(c, L.total * (size_t)rblocks, &ws))) return rc;
         if ((rc = launch_build_vpad(c, V))) return rc;

@@ -116,12 +116,45 @@ __global__ void support_mask_kernel(const uint8_t* __restrict__ ivl, int n_atoms
     }
 }
 
-int launch_support_masks(sq_ctx* ctx)
+// The most projector entries of any region row.  Every row of a node's region is
+// the middle row of some node's (periodic grid), so each node counts that one.
+__global__ void row_entries_kernel(const AtomTab* __restrict__ at, const uint8_t* __restrict__ ivl,
+                                   const int* __restrict__ tile_start, const int4* __restrict__ tile_cand, int nt0,
+                                   int nt1, int lb, int n1, int n2, long long Nd, int m, int* most)
+{
+    int best = 0;
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < Nd; q += (long long)gridDim.x * blockDim.x) {
+        const int i = (int)(q % n1), j = (int)((q / n1) % n2), k = (int)(q / ((long long)n1 * n2));
+        const int tile = i / TILE + nt0 * (j / TILE + nt1 * (k / TILE));
+        int n = 0;
+        for (int c = tile_start[tile]; c < tile_start[tile + 1]; ++c) {
+            const int4 tc = tile_cand[c];
+            const int jj = j - tc.z, kk = k - tc.w;
+            if (jj < 0 || kk < 0 || jj >= at[tc.x].len[1] || kk >= at[tc.x].len[2]) continue;
+            const uchar2 iv = *reinterpret_cast<const uchar2*>(ivl + (((size_t)tc.x * lb + jj) * lb + kk) * 2);
+            n += iv.x <= iv.y && tc.y + iv.y >= i - m && tc.y + iv.x <= i + m;
+        }
+        best = max(best, n);
+    }
+    best = __reduce_max_sync(0xffffffffu, (unsigned)best);
+    if ((threadIdx.x & 31) == 0) atomicMax(most, best);
+}
+
+// The quad kernels' support masks (ctx->d_qmask, one more word for the result of
+// the second kernel) and the most entries of any region row.  Waits.
+int launch_support_masks(sq_ctx* ctx, int* most_row_entries)
 {
     const long long n = (long long)ctx->n_atoms * ctx->lb * ctx->lb;
+    int* most = reinterpret_cast<int*>(ctx->d_qmask + n);
     support_mask_kernel<<<(int)std::min<long long>((n + 255) / 256, (long long)ctx->sm_count * 8), 256, 0, ctx->stream>>>(
         ctx->d_ivl, ctx->n_atoms, ctx->lb, ctx->d_qmask);
-    ctx->launches++;
+    SQ_CUDA_TRY(cudaMemsetAsync(most, 0, sizeof(int), ctx->stream));
+    row_entries_kernel<<<(int)std::min<long long>((ctx->g.Nd + 127) / 128, (long long)ctx->sm_count * 16), 128, 0,
+                         ctx->stream>>>(ctx->d_atoms, ctx->d_ivl, ctx->d_tile_start, ctx->d_tile_cand, ctx->ntile[0],
+                                        ctx->ntile[1], ctx->lb, ctx->g.n1, ctx->g.n2, ctx->g.Nd, ctx->g.m, most);
+    ctx->launches += 2;
+    SQ_CUDA_TRY(cudaMemcpyAsync(most_row_entries, most, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    SQ_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
 

@@ -293,6 +293,23 @@ __device__ __forceinline__ uint2 quad_entry(uint32_t x, uint32_t y, uint32_t ab,
     return make_uint2(x | (y << 14), (ab >> 2) | (nib << 16));
 }
 
+// Arguments of the quad kernels with the region arguments a.
+inline QuadArgs quad_args(const sq_ctx* c, const RegionArgs<float>& a)
+{
+    QuadArgs q;
+    memset(&q, 0, sizeof(q));
+    q.r = a;
+    for (int d = 0; d <= FD_NO; ++d) q.wd2[d] = make_float2(a.wd[d], a.wd[d]);
+    q.diag = (float)(-3.0 * c->g.w[0]);
+    q.scratch = (char*)c->d_qscratch;
+    q.stride = c->q_stride;
+    q.mask = c->d_qmask;
+    q.nxq = quad_nxq(c->lb);
+    q.nyp = quad_nyp(c->lb);
+    q.recs = quad_recs(c->lb);
+    return q;
+}
+
 // Where one CTA keeps things, and what one thread owns.
 template <int M>
 struct QuadCta {
@@ -379,8 +396,9 @@ __device__ __forceinline__ uint32_t col_mask(int xlo, int xhi) { return (0xfffff
 // tile whose box meets the region, in tile-list order), their x and y tables
 // aligned to the region's quads and row pairs, the entries (support rows) by
 // candidate for the inner products, and the lists by (quad, row pair, plane)
-// for the gather.  A region row with more than ENTRIES_PER_ROW entries is
-// reported as in the general form.  Returns the candidate count.
+// for the gather.  No region row has more than ENTRIES_PER_ROW entries (contexts
+// with such a row keep the general kernels, which refuse them).  Returns the
+// candidate count.
 template <int M>
 __device__ int quad_setup(const QuadArgs& a, const QuadCta<M>& k, int qi, int qj, int qk, int* red_i)
 {
@@ -514,19 +532,6 @@ __device__ int quad_setup(const QuadArgs& a, const QuadCta<M>& k, int qi, int qj
             if (lane == 0) k.nvis[k.sub * G::NP + zp] = most;
             for (; n < most; ++n) lp[n * 32] = none;
         }
-    }
-    // A region row with more than ENTRIES_PER_ROW entries is refused.  Every row of a node's region is the
-    // middle row of some node's (periodic grid), so each node counts that one.
-    {
-        int xlo, xhi;
-        bool in = false;
-        if (tid < ncand) {                                // at most MAX_CAND = QD_NT candidates
-            const int4 cr = k.cand[tid];
-            const int ln = k.clen[tid], jj = M - cr.z, kk = M - cr.w;
-            in = jj >= 0 && jj < ((ln >> 8) & 255) && kk >= 0 && kk < (ln >> 16) &&
-                 nl_row_interval<float, M>(nl, cr.x, cr.y, jj, kk, xlo, xhi);
-        }
-        if (__syncthreads_count(in) > ENTRIES_PER_ROW && tid == 0) atomicOr(a.r.err, ERR_CAPACITY);
     }
     // entries: warp per candidate, its box rows clipped to the region, compacted with a ballot
     for (int c = warp; c < ncand; c += QD_NW) {
@@ -948,9 +953,9 @@ __device__ void quad_stencil(const QuadArgs& a, const QuadCta<M>& k, uint32_t ca
 // The rest of a sweep with projectors: out (columns cb, the local part) += the
 // projector term, cut to the region, summed, its centre value kept.  PUB: out
 // also becomes the current vector in shared memory (every reader of the old
-// one is done).
-template <int M, bool TT, bool PUB>
-__device__ void quad_gather(const QuadCta<M>& k, uint32_t ca, uint32_t cb, QuadSums& sum, double* centre)
+// one is done).  ACCD: D += cd out, D in the owners' order (as the potential).
+template <int M, bool TT, bool PUB, bool ACCD>
+__device__ void quad_gather(const QuadCta<M>& k, uint32_t ca, uint32_t cb, QuadSums& sum, double* centre, float4* D, float cd)
 {
     using G = QGeo<M>;
     const uint32_t in = quad_inside<M>(k);
@@ -990,6 +995,12 @@ __device__ void quad_gather(const QuadCta<M>& k, uint32_t ca, uint32_t cb, QuadS
             const int z = 2 * zp + h;
             if (z >= G::S) break;                         // warp-uniform
             __syncwarp();
+            float4* dz = ACCD ? D + (size_t)((k.sub * G::S + z) * 2) * 32 + k.lane : nullptr;
+            float4 d0, d1;
+            if (ACCD) {
+                d0 = dz[0];
+                d1 = dz[32];
+            }
             float o[8], t[8];
             tm_ld8(k.tm + cb + z * 8, o);
             tm_ld8(k.tm + ca + z * 8, t);
@@ -1001,6 +1012,10 @@ __device__ void quad_gather(const QuadCta<M>& k, uint32_t ca, uint32_t cb, QuadS
             for (int i = 0; i < 8; i += 2) sum.template add<TT>(pack2(o[i], o[i + 1]), pack2(t[i], t[i + 1]));
             tm_st8(k.tm + cb + z * 8, o);
             if (!TT && z == M && k.q == M / 4 && k.p == M / 2) *centre = (double)o[(M & 1) * 4 + (M & 3)];
+            if (ACCD) {
+                dz[0] = make_float4(d0.x + cd * o[0], d0.y + cd * o[1], d0.z + cd * o[2], d0.w + cd * o[3]);
+                dz[32] = make_float4(d1.x + cd * o[4], d1.y + cd * o[5], d1.z + cd * o[6], d1.w + cd * o[7]);
+            }
             if (PUB && k.act) {
                 float* b = k.own + z * G::PL;
                 *reinterpret_cast<float4*>(b) = make_float4(o[0], o[1], o[2], o[3]);
@@ -1017,9 +1032,9 @@ __device__ void quad_gather(const QuadCta<M>& k, uint32_t ca, uint32_t cb, QuadS
 // warps begin with one and two with the other, which overlaps the stencil's FP32
 // and tensor-memory work with the loads of the inner products.  The gather
 // follows their coefficients.  sums: out.out, out.t, t.t.
-template <int M, bool TT>
+template <int M, bool TT, bool ACCD = false>
 __device__ void quad_sweep(const QuadArgs& a, const QuadCta<M>& k, uint32_t ca, uint32_t cb, float s, int ncand,
-                           float2 (*red)[QD_NW], double* centre)
+                           float2 (*red)[QD_NW], double* centre, float4* D = nullptr, float cd = 0.f)
 {
     QuadSums sum;
     if (a.r.nl.n_atoms > 0) {
@@ -1031,7 +1046,7 @@ __device__ void quad_sweep(const QuadArgs& a, const QuadCta<M>& k, uint32_t ca, 
         }
         quad_coefs<M>(a, k, ncand, s);
         tm_sync();                                        // the gather's planes are other warps' stencil planes
-        quad_gather<M, TT, !TT>(k, ca, cb, sum, centre);
+        quad_gather<M, TT, !TT, ACCD>(k, ca, cb, sum, centre, D, cd);
     } else {
         quad_stencil<M, TT, true>(a, k, ca, cb, s, sum, centre);
     }
