@@ -24,6 +24,32 @@
 
 namespace sq {
 
+// Column (x, y) or row (y, z) of a thread in the sweep and in the update: FP32
+// takes lane and warp, so that a warp's loads are one row segment; FP64, whose
+// instructions cost a warp 16 clocks of the SM however few lanes are active
+// (DFMA measured with 32, 16 and 1 of them), packs the S x S of them into as few
+// warps as hold them: 20 instead of 25 at 25^3.  With that, the slots of the inner
+// products that no lane needs left out and their four sums per candidate reduced side
+// by side, 4096 nodes of 25^3 take 477 + 273 ms (40 Lanczos steps, 24 moment steps)
+// instead of 564 + 328.
+template <typename T, int S>
+struct Owner {
+    int a, b;
+    bool on;
+    __device__ Owner()
+    {
+        if constexpr (sizeof(T) == 8) {
+            a = (int)threadIdx.x % S;
+            b = (int)threadIdx.x / S;
+            on = b < S;
+        } else {
+            a = (int)threadIdx.x & 31;
+            b = (int)threadIdx.x >> 5;
+            on = a < S;
+        }
+    }
+};
+
 template <int M>
 struct Geo {
     static constexpr int S = 2 * M + 1;
@@ -572,10 +598,18 @@ __device__ void nl_dots(const RegionArgs<T>& a, const CtaScratch<T>& sc, const T
         while (j0 + 1 >= sc.chunk_first[cB + 1]) ++cB;
         fetch(j0 + 1, cB, rB, vB);
     }
+    // slots x - bx of an entry as a bit mask
+    auto slots = [](uint32_t meta) {
+        const int xlo = (meta >> 10) & 31u, xhi = (meta >> 15) & 31u, bx = (int)((meta >> 20) & 63u) - 32;
+        return ((2u << (xhi - bx)) - 1u) & ~((1u << (xlo - bx)) - 1u);
+    };
     T aS = 0, aX = 0, aY = 0, aZ = 0;
     for (int j = j0; j < j1; ++j) {
         const EntRec<T> rc = rA;
         const bool val = vA;
+        // FP64: leave out the slots that no lane needs (a masked instruction costs as much)
+        uint32_t any = ~0u;
+        if constexpr (sizeof(T) == 8) any = __reduce_or_sync(0xffffffffu, val && unrolled ? slots(rc.meta) : 0u);
         const int c = cA;
         rA = rB;
         vA = vB;
@@ -596,10 +630,10 @@ __device__ void nl_dots(const RegionArgs<T>& a, const CtaScratch<T>& sc, const T
             const T* rowp = row + bx;
             T u = 0, u2 = 0;
             if (unrolled) {
-                const uint32_t mask = ((2u << (xhi - bx)) - 1u) & ~((1u << (xlo - bx)) - 1u);
+                const uint32_t mask = slots(rc.meta);
 #pragma unroll
                 for (int k = 0; k < LBMAX; ++k)
-                    if (mask & (1u << k)) {
+                    if ((any & (1u << k)) && (mask & (1u << k))) {
                         const P2 g = txp[k];
                         const T tv = rowp[k];
                         u += g.x * tv;
@@ -619,16 +653,28 @@ __device__ void nl_dots(const RegionArgs<T>& a, const CtaScratch<T>& sc, const T
             aZ += rc.f2 * u;
         }
         if (j + 1 >= j1 || cA != c) {                 // warp-uniform: candidate done in this warp
-            aS = warp_sumT<T>(aS);                    // xor tree: every lane holds the totals
-            aX = warp_sumT<T>(aX);
-            aY = warp_sumT<T>(aY);
-            aZ = warp_sumT<T>(aZ);
-            if (lane == 0) {
-                T* sg = sc.seg + (size_t)(c + warp) * 4;
-                sg[0] = aS;
-                sg[1] = aX;
-                sg[2] = aY;
-                sg[3] = aZ;
+            if constexpr (sizeof(T) == 8) {
+                // four sums over the warp: after two exchanges every lane works on one of them
+                const bool h = lane & 1, h2 = lane & 2;
+                const T r0 = (h ? aX : aS) + __shfl_xor_sync(0xffffffffu, h ? aS : aX, 1);
+                const T r1 = (h ? aZ : aY) + __shfl_xor_sync(0xffffffffu, h ? aY : aZ, 1);
+                T r = (h2 ? r1 : r0) + __shfl_xor_sync(0xffffffffu, h2 ? r0 : r1, 2);
+                r += __shfl_xor_sync(0xffffffffu, r, 4);
+                r += __shfl_xor_sync(0xffffffffu, r, 8);
+                r += __shfl_xor_sync(0xffffffffu, r, 16);
+                if (lane < 4) sc.seg[(size_t)(c + warp) * 4 + lane] = r;
+            } else {
+                aS = warp_sumT<T>(aS);                // xor tree: every lane holds the totals
+                aX = warp_sumT<T>(aX);
+                aY = warp_sumT<T>(aY);
+                aZ = warp_sumT<T>(aZ);
+                if (lane == 0) {
+                    T* sg = sc.seg + (size_t)(c + warp) * 4;
+                    sg[0] = aS;
+                    sg[1] = aX;
+                    sg[2] = aY;
+                    sg[3] = aZ;
+                }
             }
             aS = aX = aY = aZ = 0;
         }
@@ -684,29 +730,26 @@ __device__ inline void load_P<double>(const double* P, int c, double& pS, double
 }
 
 // sec <- sec - coef * V_nl t, candidate-ordered per point (FP64; the FP32
-// form uses nl_update_red below).  Thread (lane = y, warp = z) owns
-// region row (y, z) and walks its entries (candidates ascending); the lanes
-// of a warp take their k-th entries together, and each entry's x-interval is
-// covered by predicated slots, loads first and stores after, so every entry
-// costs a fixed, overlapped instruction sequence.  Per entry
+// form uses nl_update_red below).  A thread owns a region row and walks its
+// entries (candidates ascending); the lanes of a warp take their k-th entries
+// together.  Per entry
 //   b0 = coef (cs f0 S_c + cp (f1 Y_c + f2 Z_c)),  b1 = coef cp f0 X_c,
-// and each point of the interval gets  -= G_x b0 + DG_x b1.  The lanes own
-// neighbouring rows of one plane, whose candidates and intervals nearly
+// and each point of the interval gets  -= G_x b0 + DG_x b1: one more operation than
+// two multiply-adds onto the point, but those would wait for its load one after the
+// other (25^3, 4096 nodes: 1395 ms for bounds and moments against 750).
+// The lanes own neighbouring rows, whose candidates and intervals nearly
 // coincide, so their shared-memory accesses spread over distinct banks.
 template <typename T, int M, bool DB>
 __device__ void nl_update(const RegionArgs<T>& a, const CtaScratch<T>& sc, T* sec, T coef)
 {
     using G = Geo<M>;
     using P2 = typename Pair2<T>::type;
-    constexpr int GRP = sizeof(T) == 4 ? 5 : 4;       // slots loaded together (divides LBMAX)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool own = lane < G::S;
-    const int r = (own ? lane : 0) + G::S * warp;
-    T* brow = Sec<M, DB>::row(sec, own ? lane : 0, warp);
-    const int n = own ? sc.row_n[r] : 0;
+    const Owner<T, G::S> w;
+    const int r = w.on ? w.a + G::S * w.b : 0;
+    T* brow = Sec<M, DB>::row(sec, w.on ? w.a : 0, w.on ? w.b : 0);
+    const int n = w.on ? sc.row_n[r] : 0;
     const int nmax = __reduce_max_sync(0xffffffffu, (unsigned)n);
     if (nmax == 0) return;
-    const bool unrolled = a.nl.lb <= LBMAX;
     const T cs = a.nl.cs * coef, cp = a.nl.cp * coef;
     const P2* tx2 = reinterpret_cast<const P2*>(sc.TX);
     const EntRec<T>* rrow = sc.rec + (size_t)r * ENTRIES_PER_ROW;
@@ -729,32 +772,9 @@ __device__ void nl_update(const RegionArgs<T>& a, const CtaScratch<T>& sc, T* se
         const P2* tx = tx2 + (size_t)c * a.nl.lb + (xlo - bx);
         T* bp = brow + xlo;
         const int len = xhi - xlo;                    // slots 0..len
-        bool done = false;
-        if constexpr (sizeof(T) == 4) {               // FP64 takes the plain loop: registers matter more there
-            if (unrolled) {
-#pragma unroll
-                for (int h = 0; h < LBMAX / GRP; ++h) {
-                    if (h * GRP > len) break;
-                    P2 g[GRP];
-                    T v[GRP];
-#pragma unroll
-                    for (int s = 0; s < GRP; ++s)
-                        if (h * GRP + s <= len) {
-                            g[s] = tx[h * GRP + s];
-                            v[s] = bp[h * GRP + s];
-                        }
-#pragma unroll
-                    for (int s = 0; s < GRP; ++s)
-                        if (h * GRP + s <= len) bp[h * GRP + s] = v[s] - (g[s].x * b0 + g[s].y * b1);
-                }
-                done = true;
-            }
-        }
-        if (!done) {
-            for (int s = 0; s <= len; ++s) {
-                const P2 g = tx[s];
-                bp[s] -= g.x * b0 + g.y * b1;
-            }
+        for (int s = 0; s <= len; ++s) {
+            const P2 g = tx[s];
+            bp[s] -= g.x * b0 + g.y * b1;
         }
     }
 }
@@ -867,8 +887,9 @@ __device__ void stencil_sweep(const RegionArgs<T>& a, T* cur, T* sec, const T* v
 {
     using G = Geo<M>;
     using SV = Sec<M, DB>;
-    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
-    const bool active = x < G::S;
+    const Owner<T, G::S> own;
+    const int x = own.a, y = own.on ? own.b : 0;
+    const bool active = own.on;
     T* col = cur + G::LEAD + y * G::PX + x;
     T* bcol = SV::col(sec, x, y);
     const size_t vplane = (size_t)a.g.P1 * a.g.P2;
