@@ -132,7 +132,7 @@ def flops_lanczos(wl):
 # the sources that define the region kernels (their counters are recorded
 # against this hash, so any change to these files voids them)
 KERNEL_SOURCES = ("sq_internal.cuh", "sq_region.cuh", "sq_region_dispatch.cuh", "sq_region_f32.cu",
-                  "sq_region_f64.cu")
+                  "sq_region_f64.cu", "sq_quad.cuh", "sq_quad.cu")
 
 
 def source_sha():
