@@ -735,6 +735,7 @@ def run_force(a):
     t = float(np.mean(times))
     nt = touched_nodes(wl, s.positions)
     S = 2 * wl.m + 1
+    quad = prec == SQ_FP32 and 7 <= wl.m <= 15 and not os.environ.get("SQ_FORCE_KERNEL")    # the form that runs by default
     units = nt * wl.npl
     flops = nt * wl.npl * S ** 3 * (FORCE_FLOPS_PER_POINT + NL_FLOPS_PER_PAIR * nl_pairs_per_point(wl))
     peaks = json.load(open(PEAKS_PATH)) if os.path.exists(PEAKS_PATH) else {}
@@ -760,12 +761,13 @@ def run_force(a):
                               if os.environ.get("SQ_FORCE_KERNEL") == "legacy" and os.environ.get("SQ_FORCE_SMEM") == "1"
                               else "first form, vectors in global scratch (SQ_FORCE_KERNEL=legacy)"
                               if os.environ.get("SQ_FORCE_KERNEL") == "legacy"
+                              else "quad form (the quad kernels' recurrence with D in global scratch)" if quad
                               else "region form (the region kernels' recurrence with D in global scratch)"),
                    "l2": "flushed between timed steps (256 MB write)",
                    "parallelism": "single GPU"},
         "forces_max_abs": float(F.abs().max().item()),
         "roofline": {"kernel": ("nl_force_kernel" if os.environ.get("SQ_FORCE_KERNEL") == "legacy"
-                                else "force_region_kernel"),
+                                else "quad_force_kernel" if quad else "force_region_kernel"),
                      "bound": "alu", "achieved": flops / t / 1e12, "peak": peak,
                      "unit": "TFLOP/s", "frac": flops / t / 1e12 / peak, "traffic": None, "peak_basis": basis},
         "e2e": {"value": units / float(np.median(e2e)), "unit": FORCE_UNIT,
