@@ -42,6 +42,7 @@ struct Owner {
             a = (int)threadIdx.x % S;
             b = (int)threadIdx.x / S;
             on = b < S;
+            if (!on) b = 0;
         } else {
             a = (int)threadIdx.x & 31;
             b = (int)threadIdx.x >> 5;
@@ -608,7 +609,7 @@ __device__ void nl_dots(const RegionArgs<T>& a, const CtaScratch<T>& sc, const T
         const EntRec<T> rc = rA;
         const bool val = vA;
         // FP64: leave out the slots that no lane needs (a masked instruction costs as much)
-        uint32_t any = ~0u;
+        [[maybe_unused]] uint32_t any = 0;
         if constexpr (sizeof(T) == 8) any = __reduce_or_sync(0xffffffffu, val && unrolled ? slots(rc.meta) : 0u);
         const int c = cA;
         rA = rB;
@@ -630,10 +631,10 @@ __device__ void nl_dots(const RegionArgs<T>& a, const CtaScratch<T>& sc, const T
             const T* rowp = row + bx;
             T u = 0, u2 = 0;
             if (unrolled) {
-                const uint32_t mask = slots(rc.meta);
+                const uint32_t mask = ((2u << (xhi - bx)) - 1u) & ~((1u << (xlo - bx)) - 1u);
 #pragma unroll
                 for (int k = 0; k < LBMAX; ++k)
-                    if ((any & (1u << k)) && (mask & (1u << k))) {
+                    if ((sizeof(T) == 4 || (any & (1u << k))) && (mask & (1u << k))) {
                         const P2 g = txp[k];
                         const T tv = rowp[k];
                         u += g.x * tv;
@@ -888,7 +889,7 @@ __device__ void stencil_sweep(const RegionArgs<T>& a, T* cur, T* sec, const T* v
     using G = Geo<M>;
     using SV = Sec<M, DB>;
     const Owner<T, G::S> own;
-    const int x = own.a, y = own.on ? own.b : 0;
+    const int x = own.a, y = own.b;
     const bool active = own.on;
     T* col = cur + G::LEAD + y * G::PX + x;
     T* bcol = SV::col(sec, x, y);
