@@ -484,14 +484,27 @@ int sq_sync(sq_ctx *ctx);
 /* Number of kernel launches this context has enqueued since creation. */
 long long sq_launch_count(const sq_ctx *ctx);
 
+/* Forms of the region kernels, as sq_context_info reports them. */
+enum {
+    SQ_FORM_NONE = -1,      /* no kernel (no projectors: no forces)               */
+    SQ_FORM_GENERAL = 0,    /* one CTA per node, either precision, every size     */
+    SQ_FORM_CLUSTER = 1,    /* FP32, thread-block clusters (SQ_REGION_KERNEL=cluster) */
+    SQ_FORM_QUAD = 2,       /* FP32, quads of points per thread                   */
+    SQ_FORM_FIRST = 3       /* forces only: every vector in global scratch        */
+};
+
 /* Launch configuration the context chose (host only, no synchronisation).
- * info_host: HOST array of n >= 4 ints receiving
+ * info_host: HOST array of n >= 4 ints; the first min(n, 7) receive
  *   [0] m, the region half-width in grid points (region side 2m+1);
  *   [1] the largest number of projector candidates of any node;
- *   [2] where the per-candidate projector tables live during the region
- *       kernels: 0 global scratch, 1 all in shared memory, 2 the tables every
- *       step reads in shared memory and the rest in global scratch;
- *   [3] resident CTAs of the region kernels (per-CTA scratch slices).
+ *   [2] where the per-candidate projector tables live during the general
+ *       region kernels: 0 global scratch, 1 all in shared memory, 2 the tables
+ *       every step reads in shared memory and the rest in global scratch;
+ *   [3] resident CTAs of the general region kernels (per-CTA scratch slices);
+ *   [4] the form that sq_spectral_bounds runs (SQ_FORM_*);
+ *   [5] the form that sq_moments runs;
+ *   [6] the form that sq_nl_forces runs now (SQ_FORCE_KERNEL is read on every
+ *       call).
  * SQ_EINVAL for a NULL context or n < 4. */
 int sq_context_info(const sq_ctx *ctx, int *info_host, int n);
 

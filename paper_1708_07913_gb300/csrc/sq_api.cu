@@ -1108,6 +1108,9 @@ int sq_context_info(const sq_ctx* c, int* info, int n)
     info[1] = c->ccap;
     info[2] = c->nl_mode;
     info[3] = c->grid_blocks;
+    for (int i = 4; i < n && i < 6; ++i)
+        info[i] = c->cl_nc > 0 ? SQ_FORM_CLUSTER : c->quad[i == 4 ? 1 : 0] ? SQ_FORM_QUAD : SQ_FORM_GENERAL;
+    if (n > 6) info[6] = force_form(c);
     return SQ_OK;
 }
 

@@ -207,7 +207,7 @@ RegionForceLayout region_force_layout(int S, int n_atoms, size_t tsz)
 }
 
 // Grid of the region form (0: not available for this context).
-int region_force_blocks(sq_ctx* c, long long nq, size_t* extra)
+int region_force_blocks(const sq_ctx* c, long long nq, size_t* extra)
 {
     if (c->cl_nc > 0 || !c->d_scratch) return 0;        // the cluster kernels keep no per-CTA scratch
     const char* env = getenv("SQ_FORCE_KERNEL");
@@ -257,7 +257,7 @@ int launch_force_region(sq_ctx* c, const RegionForceLayout& L, char* base, int b
 }
 
 // Grid of the quad form (0: not available for this context).
-int quad_force_blocks(sq_ctx* c, long long nq, size_t* smem)
+int quad_force_blocks(const sq_ctx* c, long long nq, size_t* smem)
 {
     const char* env = getenv("SQ_FORCE_KERNEL");
     if (!c->quad[0] || (env && (strcmp(env, "legacy") == 0 || strcmp(env, "region") == 0))) return 0;
@@ -352,6 +352,14 @@ void free_force_ws(sq_ctx* c)
     if (it == g_force_ws.end()) return;
     ws_release(it->second);
     g_force_ws.erase(it);
+}
+
+int force_form(const sq_ctx* c)
+{
+    size_t extra = 0;
+    if (c->n_atoms == 0 || (!c->has_s && !c->has_p)) return SQ_FORM_NONE;
+    if (quad_force_blocks(c, c->g.Nd, &extra) > 0) return SQ_FORM_QUAD;
+    return region_force_blocks(c, c->g.Nd, &extra) > 0 ? SQ_FORM_GENERAL : SQ_FORM_FIRST;
 }
 }  // namespace sq
 

@@ -202,6 +202,7 @@ constexpr int FERMI_STATE = 12;      // doubles of the device Fermi/energy state
 int fermi_result(const double* st_host, double* mu, double* eb, double* es, double* ne);
 int launch_proj_tables(sq_ctx* ctx, const double* d_R);
 int launch_support_masks(sq_ctx* ctx, int* most_row_entries);
+int force_form(const sq_ctx* ctx);       // SQ_FORM_* that nl_forces runs
 }  // namespace sq
 
 #define SQ_CUDA_TRY(call)                                   \

@@ -226,15 +226,19 @@ def sq_launch_count(ctx) -> int:
 
 
 NL_GLOBAL, NL_ALL, NL_HOT = 0, 1, 2
+FORM_NONE, FORM_GENERAL, FORM_CLUSTER, FORM_QUAD, FORM_FIRST = -1, 0, 1, 2, 3
 
 
 def sq_context_info(ctx) -> dict:
     """The launch configuration the context chose: region half-width m, the
-    most projector candidates of any node, the projector-table placement
-    (NL_GLOBAL / NL_ALL / NL_HOT) and the region kernels' resident CTAs."""
-    out = (C.c_int * 4)()
-    _check(load().sq_context_info(C.c_void_p(ctx), out, 4), "sq_context_info")
-    return dict(m=out[0], ccap=out[1], tables=out[2], blocks=out[3])
+    most projector candidates of any node, the general region kernels'
+    projector-table placement (NL_GLOBAL / NL_ALL / NL_HOT) and resident CTAs,
+    and the form of the Lanczos, moments and force kernels that run
+    (FORM_GENERAL / FORM_CLUSTER / FORM_QUAD, forces also FORM_FIRST or, without
+    projectors, FORM_NONE)."""
+    out = (C.c_int * 7)()
+    _check(load().sq_context_info(C.c_void_p(ctx), out, 7), "sq_context_info")
+    return dict(m=out[0], ccap=out[1], tables=out[2], blocks=out[3], lanczos=out[4], moments=out[5], forces=out[6])
 
 
 def sq_destroy(ctx):
