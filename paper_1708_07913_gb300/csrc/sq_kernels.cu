@@ -464,8 +464,11 @@ __global__ void fermi_bracket_kernel(const double* __restrict__ chi, const doubl
 // First zero k with chi + zeta x_k - mu <= 41 kT, or up to two before it (x_k
 // falls with k, FP32, the margin covers its rounding): where the terms begin
 // that are not 0.  With the sign of the bound turned, past which they are 1.
+// An interval run through backwards or of one point (z <= 0) has no such order:
+// every zero is visited.
 __device__ inline int zero_index(double c, double z, double bound, int K, bool up)
 {
+    if (!(z > 0.0)) return up ? K : 0;
     const float x = fminf(1.0f, fmaxf(-1.0f, (float)(bound - c) / (float)z));
     const float k = acosf(x) * (float)K * 0.318309886f - 0.5f;
     const int i = up ? (int)ceilf(k) + 1 : (int)floorf(k) - 1;
