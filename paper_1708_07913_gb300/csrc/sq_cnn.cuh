@@ -467,6 +467,11 @@ __global__ void __launch_bounds__(CNN_NT) cnn_out_bwd_kernel(CnnGrid g, const fl
 // extra tap K^3 is the bias (A = 1, input 0).  Tiles of 8 x 8 x 2 nodes, A with
 // its neighbours and G in shared memory (zero beyond the grid); rows of 8 nodes
 // along x share the loads of A between the taps dx and those of G between dy.
+// Every tile's sums are added to part by themselves: FP32 chains of 128 nodes and
+// then of tiles (171 at 128^3), not of all the block's nodes (21,888 there).  The
+// additions are reductions that nothing waits for (a gradient at 64^3, one sample:
+// 1.86 ms with one chain per block, 1.99 with the sums read back, 1.88 so); one
+// thread's reductions of one address keep their order.
 // 16^3 nodes: a block per (4096 nodes, tap), each node in turn, took 464 us for the
 // middle layer, 374 for the last and 898 for the first; these take 21, 20 and 11.
 constexpr int WG_X = 8, WG_Y = 8, WG_Z = 2;
@@ -484,11 +489,7 @@ __global__ void __launch_bounds__(CNN_NT) cnn_wgrad2_kernel(CnnGrid g, const flo
     float* sA = wsm2 + OWN * CNN_C;                      // [node][33]
     const int in = threadIdx.x & 31, oq = threadIdx.x >> 5;
     const int dz = (int)blockIdx.y - 1;
-    float acc[9][4], bias[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-    for (int d = 0; d < 9; ++d)
-#pragma unroll
-        for (int o = 0; o < 4; ++o) acc[d][o] = 0.0f;
+    float* out = part + (size_t)blockIdx.x * 28 * CNN_C * CNN_C;
     const long long nt = cnn_tiles<WG_X, WG_Y, WG_Z>(g);
     for (long long t = blockIdx.x; t < nt; t += gridDim.x) {
         const CnnTile c = cnn_tile<WG_X, WG_Y, WG_Z>(g, t);
@@ -505,6 +506,11 @@ __global__ void __launch_bounds__(CNN_NT) cnn_wgrad2_kernel(CnnGrid g, const flo
                         ? G[((long long)px + (long long)g.n1 * (py + (long long)g.n2 * pz)) * CNN_C + ch] : 0.0f;
         }
         __syncthreads();
+        float acc[9][4], bias[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int d = 0; d < 9; ++d)
+#pragma unroll
+            for (int o = 0; o < 4; ++o) acc[d][o] = 0.0f;
         for (int r = 0; r < WG_Y * WG_Z; ++r) {
             const int ly = r % WG_Y, lz = r / WG_Y;
             float4 gv[WG_X];
@@ -535,14 +541,16 @@ __global__ void __launch_bounds__(CNN_NT) cnn_wgrad2_kernel(CnnGrid g, const flo
                     }
             }
         }
-    }
-    float* out = part + (size_t)blockIdx.x * 28 * CNN_C * CNN_C;
+        const bool first = t == blockIdx.x;
+        auto add = [&](float* to, const float (&v)[4]) {
+            if (first) *reinterpret_cast<float4*>(to) = make_float4(v[0], v[1], v[2], v[3]);
+            else asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};"
+                              ::"l"(to), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+        };
 #pragma unroll
-    for (int d = 0; d < 9; ++d)
-        *reinterpret_cast<float4*>(out + ((size_t)((dz + 1) * 9 + d) * CNN_C + in) * CNN_C + 4 * oq) =
-            make_float4(acc[d][0], acc[d][1], acc[d][2], acc[d][3]);
-    if (dz == 0 && in == 0)
-        *reinterpret_cast<float4*>(out + (size_t)27 * CNN_C * CNN_C + 4 * oq) = make_float4(bias[0], bias[1], bias[2], bias[3]);
+        for (int d = 0; d < 9; ++d) add(out + ((size_t)((dz + 1) * 9 + d) * CNN_C + in) * CNN_C + 4 * oq, acc[d]);
+        if (dz == 0 && in == 0) add(out + (size_t)27 * CNN_C * CNN_C + 4 * oq, bias);
+    }
 }
 
 // First layer (1 -> 32, 5^3 taps): a lane per output, a warp per group of (dz, dy) rows of taps.
@@ -553,11 +561,7 @@ __global__ void __launch_bounds__(CNN_NT) cnn_wgrad1_kernel(CnnGrid g, const flo
     constexpr int PX = WG_X + 4, PY = WG_Y + 4, PZ = WG_Z + 4, OWN = WG_X * WG_Y * WG_Z, NG = CNN_NT / 32;
     __shared__ __align__(16) float sG[OWN * CNN_C], sA[PX * PY * PZ];
     const int o = threadIdx.x & 31, grp = threadIdx.x >> 5;
-    float acc[4][5], bias = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int d = 0; d < 5; ++d) acc[i][d] = 0.0f;
+    float* out = part + (size_t)blockIdx.x * 126 * CNN_C;
     const long long nt = cnn_tiles<WG_X, WG_Y, WG_Z>(g);
     for (long long t = blockIdx.x; t < nt; t += gridDim.x) {
         const CnnTile c = cnn_tile<WG_X, WG_Y, WG_Z>(g, t);
@@ -571,6 +575,11 @@ __global__ void __launch_bounds__(CNN_NT) cnn_wgrad1_kernel(CnnGrid g, const flo
                         ? G[((long long)px + (long long)g.n1 * (py + (long long)g.n2 * pz)) * CNN_C + ch] : 0.0f;
         }
         __syncthreads();
+        float acc[4][5], bias = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int d = 0; d < 5; ++d) acc[i][d] = 0.0f;
         for (int r = 0; r < WG_Y * WG_Z; ++r) {
             const int ly = r % WG_Y, lz = r / WG_Y;
             float gv[WG_X];
@@ -594,14 +603,18 @@ __global__ void __launch_bounds__(CNN_NT) cnn_wgrad1_kernel(CnnGrid g, const flo
                 }
             }
         }
+        const bool first = t == blockIdx.x;
+        auto add = [&](float* to, float v) {
+            if (first) *to = v;
+            else asm volatile("red.global.add.f32 [%0], %1;" ::"l"(to), "f"(v) : "memory");
+        };
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (grp + NG * i < 25)
+#pragma unroll
+                for (int dx = 0; dx < 5; ++dx) add(out + ((grp + NG * i) * 5 + dx) * CNN_C + o, acc[i][dx]);
+        if (grp == 0) add(out + 125 * CNN_C + o, bias);
     }
-    float* out = part + (size_t)blockIdx.x * 126 * CNN_C;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        if (grp + NG * i < 25)
-#pragma unroll
-            for (int dx = 0; dx < 5; ++dx) out[((grp + NG * i) * 5 + dx) * CNN_C + o] = acc[i][dx];
-    if (grp == 0) out[125 * CNN_C + o] = bias;
 }
 
 // Output layer (32 -> 1, 3^3 taps): a lane per input, a warp per row of taps; the
@@ -615,7 +628,7 @@ __global__ void __launch_bounds__(CNN_NT) cnn_wgrad3_kernel(CnnGrid g, const flo
     float* sA = wsm3;                                    // [node][32]
     float* sG = wsm3 + PX * PY * PZ * CNN_C;
     const int in = threadIdx.x & 31, grp = threadIdx.x >> 5;
-    float acc[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}}, bias = 0.0f;
+    float* out = part + (size_t)blockIdx.x * 28 * CNN_C;
     const long long nt = cnn_tiles<WG_X, WG_Y, WG_Z>(g);
     for (long long t = blockIdx.x; t < nt; t += gridDim.x) {
         const CnnTile c = cnn_tile<WG_X, WG_Y, WG_Z>(g, t);
@@ -630,6 +643,7 @@ __global__ void __launch_bounds__(CNN_NT) cnn_wgrad3_kernel(CnnGrid g, const flo
             sG[n] = px < g.n1 && py < g.n2 && pz < g.n3 ? G[(long long)px + (long long)g.n1 * (py + (long long)g.n2 * pz)] : 0.0f;
         }
         __syncthreads();
+        float acc[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}}, bias = 0.0f;
         for (int r = 0; r < WG_Y * WG_Z; ++r) {
             const int ly = r % WG_Y, lz = r / WG_Y;
             float gv[WG_X];
@@ -653,14 +667,18 @@ __global__ void __launch_bounds__(CNN_NT) cnn_wgrad3_kernel(CnnGrid g, const flo
                 }
             }
         }
+        const bool first = t == blockIdx.x;
+        auto add = [&](float* to, float v) {
+            if (first) *to = v;
+            else asm volatile("red.global.add.f32 [%0], %1;" ::"l"(to), "f"(v) : "memory");
+        };
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (grp + NG * i < 9)
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) add(out + ((grp + NG * i) * 3 + dx) * CNN_C + in, acc[i][dx]);
+        if (grp == 0) add(out + 27 * CNN_C + in, in == 0 ? bias : 0.0f);
     }
-    float* out = part + (size_t)blockIdx.x * 28 * CNN_C;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-        if (grp + NG * i < 9)
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx) out[((grp + NG * i) * 3 + dx) * CNN_C + in] = acc[i][dx];
-    if (grp == 0) out[27 * CNN_C + in] = in == 0 ? bias : 0.0f;
 }
 constexpr size_t WG3_SMEM = ((size_t)(WG_X + 2) * (WG_Y + 2) * (WG_Z + 2) * CNN_C + WG_X * WG_Y * WG_Z) * sizeof(float);
 
