@@ -133,10 +133,13 @@ int sq_moments(sq_ctx *ctx, const double *V, const double *chi, const double *ze
 
 /* Fermi level (Section 3.2): solve 2 sum_q sum_j c_q^j(mu) rho_q^j = N_e with
  * c_q^j the Chebyshev coefficients of the Fermi-Dirac function (Eq. cqj) by
- * discrete orthogonality at the npl+1 zeros of T_{npl+1}.  Bisection on
- * [min(chi-zeta) - 10 kT, max(chi+zeta) + 10 kT] until the midpoint equals an
- * end point in FP64 (at most 200 steps).  Also stores the quadrature weights
- * W_qk in the context for sq_density_energy.
+ * discrete orthogonality at the npl+1 zeros of T_{npl+1}.  A bracketing search
+ * on [min(chi-zeta) - 10 kT, max(chi+zeta) + 10 kT]: every pass counts the
+ * electrons at one to seven points inside the bracket (one to three levels of
+ * bisection, or points around the secant once it is narrower than kT/4) and so
+ * at least halves it, until its midpoint equals an end point in FP64 (at most
+ * 200 passes); mu is the midpoint.  The quadrature weights W_qk stay in the
+ * context's workspace.
  *   moments, chi, zeta   device, as produced above
  *   n_electrons          0 < N_e < 2 N_d
  *   kT                   smearing sigma > 0, Ha

@@ -392,6 +392,7 @@ __device__ inline void block_reduce(double (&v)[NV], double* sh)
 enum { F_LO = 0, F_HI, F_NE, F_KT, F_NLO, F_NHI, F_DONE, F_ITERS, F_STATUS, F_EB, F_ES, F_NEL, F_NSTATE,
        F_FINE = 12, F_NPTS, F_PTS };
 constexpr int FERMI_PTS = 7;
+constexpr int FERMI_MAX = 200;                            // passes of a search, at most
 static_assert(F_NSTATE == FERMI_STATE && F_PTS + FERMI_PTS <= 32, "Fermi state size");
 
 // Sum of one value per thread over the partials of all blocks, by the whole of
@@ -468,11 +469,10 @@ __global__ void fermi_bracket_kernel(const double* __restrict__ chi, const doubl
 // every zero is visited.
 __device__ inline int zero_index(double c, double z, double bound, int K, bool up)
 {
-    if (!(z > 0.0)) return up ? K : 0;
-    const float x = fminf(1.0f, fmaxf(-1.0f, (float)(bound - c) / (float)z));
+    const float zf = (float)z, x = fminf(1.0f, fmaxf(-1.0f, (float)(bound - c) / zf));
     const float k = acosf(x) * (float)K * 0.318309886f - 0.5f;
     const int i = up ? (int)ceilf(k) + 1 : (int)floorf(k) - 1;
-    return min(K, max(0, i));
+    return zf > 0.0f ? min(K, max(0, i)) : up ? K : 0;
 }
 
 // The next points of the search (thread 0).  lo < hi bracket the electron
@@ -524,89 +524,10 @@ __device__ void fermi_next(double* st, double lo, double hi, double fl, double f
     st[F_FINE] = fine ? 1.0 : 0.0;
 }
 
-// Electron count N(mu) = 2 sum_q sum_k W_qk g((chi_q + zeta_q x_k - mu)/kT) at
-// up to FERMI_PTS points at once, then (last block) the bracket they leave and
-// the next points.  Beyond |t| = 40 the Fermi factor is 1.0 exactly in FP64
-// (t < -40) or below 4.3e-18 (t > 40, dropped: < 1e-16 of any count here), so a
-// node visits only the zeros around mu.  What bounds it is FP64 (two lanes per
-// clock and SM): a term is an exponential and a division; within a bracket far
-// narrower than kT the points share the exponential, e^{(E-mu)/kT} = a s.  The
-// level, density and energies of 64^3 nodes at n_pl 48 took 31.8 ms with about
-// 60 bisection passes that each visited every zero, one node's row per thread,
-// and take 7.5 ms now.
-__global__ void fermi_search_kernel(const double* __restrict__ W, const double* __restrict__ chi,
-                                    const double* __restrict__ zeta, long long Nd, int K, int coarse, double* red,
-                                    unsigned* count, double* st)
+// The bracket that the counts acc at the points leave, and the next points (thread 0).
+__device__ void fermi_decide(double* st, const double (&acc)[FERMI_PTS], const double* pts, int np, bool fine, int coarse)
 {
-    __shared__ double sh[FERMI_PTS * 32];
-    __shared__ bool last;
-    __shared__ double xk[MAX_NPL + 1], pts[FERMI_PTS], sc[FERMI_PTS];
-    if (st[F_DONE] != 0.0) return;                        // uniform over the grid
-    const double kT = st[F_KT];
-    const int np = (int)st[F_NPTS];
-    const bool fine = st[F_FINE] > 0.5;
-    const double ref = st[F_PTS + (np >> 1)];
-    for (int k = threadIdx.x; k < K; k += blockDim.x) xk[k] = cos(M_PI * (k + 0.5) / K);
-    if ((int)threadIdx.x < np) {
-        pts[threadIdx.x] = st[F_PTS + threadIdx.x];
-        sc[threadIdx.x] = fine ? exp((ref - st[F_PTS + threadIdx.x]) / kT) : 0.0;
-    }
-    __syncthreads();
-    double acc[FERMI_PTS];
-#pragma unroll
-    for (int i = 0; i < FERMI_PTS; ++i) acc[i] = 0.0;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < Nd;
-         q += (long long)gridDim.x * blockDim.x) {
-        const double c = chi[q], z = zeta[q];
-        const double* w = W + q;
-        if (fine) {
-            const int ka = zero_index(c, z, pts[np - 1] + 41.0 * kT, K, false);
-            const int kb = zero_index(c, z, pts[0] - 41.0 * kT, K, true);
-            double s[FERMI_PTS], full = 0.0;
-#pragma unroll
-            for (int i = 0; i < FERMI_PTS; ++i) s[i] = 0.0;
-            for (int k = ka; k < kb; ++k) {
-                const double wk = w[(long long)k * Nd], a = exp((c + z * xk[k] - ref) / kT);
-#pragma unroll
-                for (int i = 0; i < FERMI_PTS; ++i)
-                    if (i < np) s[i] += wk / (1.0 + a * sc[i]);
-            }
-            for (int k = max(ka, kb); k < K; ++k) full += w[(long long)k * Nd];
-#pragma unroll
-            for (int i = 0; i < FERMI_PTS; ++i)
-                if (i < np) acc[i] += 2.0 * (s[i] + full);
-        } else {
-#pragma unroll
-            for (int i = 0; i < FERMI_PTS; ++i) {
-                if (i >= np) break;
-                const double mu = pts[i];
-                const int ka = zero_index(c, z, mu + 41.0 * kT, K, false);
-                const int kb = zero_index(c, z, mu - 41.0 * kT, K, true);
-                double s = 0.0;
-                for (int k = ka; k < kb; ++k) {
-                    const double t = (c + z * xk[k] - mu) / kT;
-                    if (t > 40.0) continue;
-                    const double wk = w[(long long)k * Nd];
-                    s += (t < -40.0) ? wk : wk / (1.0 + exp(t));
-                }
-                for (int k = max(ka, kb); k < K; ++k) s += w[(long long)k * Nd];
-                acc[i] += 2.0 * s;
-            }
-        }
-    }
-    block_reduce<FERMI_PTS>(acc, sh);
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < FERMI_PTS; ++i) red[(size_t)FERMI_PTS * blockIdx.x + i] = acc[i];
-        __threadfence();
-        last = atomicAdd(count, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    sum_partials<FERMI_PTS>(red, gridDim.x, acc, sh);
-    if (threadIdx.x != 0) return;
     const double Ne = st[F_NE];
-    *count = 0;
     if (st[F_FINE] < -0.5) {                              // the ends
         if (!(acc[0] <= Ne && acc[1] >= Ne)) {
             st[F_NLO] = acc[0];
@@ -638,6 +559,99 @@ __global__ void fermi_search_kernel(const double* __restrict__ W, const double* 
     }
     st[F_ITERS] += 1.0;
     fermi_next(st, lo, hi, fl, fh, coarse);
+    if (st[F_ITERS] >= FERMI_MAX) st[F_DONE] = 1.0;
+}
+
+// Electron count N(mu) = 2 sum_q sum_k W_qk g((chi_q + zeta_q x_k - mu)/kT) at
+// up to FERMI_PTS points at once, then (last block) the bracket they leave and
+// the next points.  Beyond |t| = 40 the Fermi factor is 1.0 exactly in FP64
+// (t < -40) or below 4.3e-18 (t > 40, dropped: < 1e-16 of any count here), so a
+// node visits only the zeros around mu.  What bounds it is FP64 (two lanes per
+// clock and SM): a term is an exponential and a division; within a bracket far
+// narrower than kT the points share the exponential, e^{(E-mu)/kT} = a s.  The
+// level, density and energies of 64^3 nodes at n_pl 48 took 31.8 ms with about
+// 60 bisection passes that each visited every zero, one node's row per thread,
+// and take 7.5 ms now.
+template <bool MANY>
+__global__ void fermi_search_kernel(const double* __restrict__ W, const double* __restrict__ chi,
+                                    const double* __restrict__ zeta, long long Nd, int K, int coarse, int rounds,
+                                    double* red, unsigned* count, double* st)
+{
+    __shared__ double sh[FERMI_PTS * 32];
+    __shared__ bool last;
+    __shared__ double xk[MAX_NPL + 1], pts[FERMI_PTS], sc[FERMI_PTS];
+    if (st[F_DONE] != 0.0) return;                        // uniform over the grid
+    for (int k = threadIdx.x; k < K; k += blockDim.x) xk[k] = cos(M_PI * (k + 0.5) / K);
+    for (int round = 0; round < (MANY ? rounds : 1); ++round) {      // MANY: a grid of one block
+        const double kT = st[F_KT];
+        const int np = (int)st[F_NPTS];
+        const bool fine = st[F_FINE] > 0.5;
+        const double ref = st[F_PTS + (np >> 1)];
+        if ((int)threadIdx.x < np) {
+            pts[threadIdx.x] = st[F_PTS + threadIdx.x];
+            sc[threadIdx.x] = fine ? exp((ref - st[F_PTS + threadIdx.x]) / kT) : 0.0;
+        }
+        __syncthreads();
+        double acc[FERMI_PTS];
+#pragma unroll
+        for (int i = 0; i < FERMI_PTS; ++i) acc[i] = 0.0;
+        for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < Nd;
+             q += (long long)gridDim.x * blockDim.x) {
+            const double c = chi[q], z = zeta[q];
+            const double* w = W + q;
+            if (fine) {
+                const int ka = zero_index(c, z, pts[np - 1] + 41.0 * kT, K, false);
+                const int kb = zero_index(c, z, pts[0] - 41.0 * kT, K, true);
+                double s[FERMI_PTS], full = 0.0;
+#pragma unroll
+                for (int i = 0; i < FERMI_PTS; ++i) s[i] = 0.0;
+                for (int k = ka; k < kb; ++k) {
+                    const double wk = w[(long long)k * Nd], a = exp((c + z * xk[k] - ref) / kT);
+#pragma unroll
+                    for (int i = 0; i < FERMI_PTS; ++i)
+                        if (i < np) s[i] += wk / (1.0 + a * sc[i]);
+                }
+                for (int k = max(ka, kb); k < K; ++k) full += w[(long long)k * Nd];
+#pragma unroll
+                for (int i = 0; i < FERMI_PTS; ++i)
+                    if (i < np) acc[i] += 2.0 * (s[i] + full);
+            } else {
+#pragma unroll
+                for (int i = 0; i < FERMI_PTS; ++i) {
+                    if (i >= np) break;
+                    const double mu = pts[i];
+                    const int ka = zero_index(c, z, mu + 41.0 * kT, K, false);
+                    const int kb = zero_index(c, z, mu - 41.0 * kT, K, true);
+                    double s = 0.0;
+                    for (int k = ka; k < kb; ++k) {
+                        const double t = (c + z * xk[k] - mu) / kT;
+                        if (t > 40.0) continue;
+                        const double wk = w[(long long)k * Nd];
+                        s += (t < -40.0) ? wk : wk / (1.0 + exp(t));
+                    }
+                    for (int k = max(ka, kb); k < K; ++k) s += w[(long long)k * Nd];
+                    acc[i] += 2.0 * s;
+                }
+            }
+        }
+        block_reduce<FERMI_PTS>(acc, sh);
+        if (threadIdx.x == 0) {
+            for (int i = 0; i < FERMI_PTS; ++i) red[(size_t)FERMI_PTS * blockIdx.x + i] = acc[i];
+            __threadfence();
+            last = atomicAdd(count, 1u) == gridDim.x - 1;
+        }
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        sum_partials<FERMI_PTS>(red, gridDim.x, acc, sh);
+        if (threadIdx.x == 0) {
+            *count = 0;
+            fermi_decide(st, acc, pts, np, fine, coarse);
+        }
+        if (!MANY) return;
+        __syncthreads();
+        if (st[F_DONE] != 0.0) return;
+    }
 }
 
 // Search state reset (a kernel rather than a host copy, so the whole
@@ -658,14 +672,19 @@ static int node_blocks(const sq_ctx* ctx, int threads)
     return (int)std::min<long long>((ctx->g.Nd + threads - 1) / threads, ctx->red_blocks);
 }
 
-static int enqueue_search(sq_ctx* ctx, const double* chi, const double* zeta, int launches)
+// Launches of one pass each over the whole GPU; one block that makes all the passes left.
+static int enqueue_search(sq_ctx* ctx, const double* chi, const double* zeta, int launches, bool one_block = false)
 {
     const int T = node_threads(ctx->g.Nd, ctx->sm_count), B = node_blocks(ctx, T);
     // far from the level a large system takes one point per pass (FP64-bound), a small one three (launch-bound)
     const int coarse = ctx->g.Nd >= 65536 ? 1 : 3;
+    auto launch = [&](auto kernel, int blocks, int threads) {
+        kernel<<<blocks, threads, 0, ctx->stream>>>(ctx->d_W, chi, zeta, ctx->g.Nd, ctx->npl + 1, coarse, FERMI_MAX,
+                                                    ctx->d_red, ctx->d_count, ctx->d_fermi);
+    };
     for (int it = 0; it < launches; ++it)
-        fermi_search_kernel<<<B, T, 0, ctx->stream>>>(ctx->d_W, chi, zeta, ctx->g.Nd, ctx->npl + 1, coarse, ctx->d_red,
-                                                      ctx->d_count, ctx->d_fermi);
+        if (one_block) launch(fermi_search_kernel<true>, 1, RED_T);
+        else launch(fermi_search_kernel<false>, B, T);
     ctx->launches += launches;
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
@@ -680,9 +699,12 @@ static int enqueue_search_start(sq_ctx* ctx, const double* chi, const double* ze
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
 
-// Passes that always end the search: bisection alone to kT/4 (at most 1e9 times
-// narrower than the spectrum for one point per pass) and to the last bit of FP64
-// after that; the passes past its end return at once.
+// A pass at least halves the bracket, and the search ends when its midpoint equals
+// an end point: after 53 + log2(spectrum / |mu|) halvings or so where the count is
+// flat around mu, and after 20 to 45 passes otherwise.  Passes past the end return
+// at once.  A caller that waits queues lots of FERMI_FIRST until the search says
+// that it has ended; a captured search queues FERMI_PASSES, and the rest (hardly
+// ever any) are made by one block, which needs no further launches.
 constexpr int FERMI_PASSES = 56, FERMI_FIRST = 18;
 
 // Enqueue the whole Fermi-level search on ctx->stream (no host wait); the
@@ -690,8 +712,9 @@ constexpr int FERMI_PASSES = 56, FERMI_FIRST = 18;
 // in st[F_STATUS].
 int enqueue_fermi(sq_ctx* ctx, const double* chi, const double* zeta, double Ne, double kT)
 {
-    const int rc = enqueue_search_start(ctx, chi, zeta, Ne, kT);
-    return rc ? rc : enqueue_search(ctx, chi, zeta, FERMI_PASSES);
+    int rc = enqueue_search_start(ctx, chi, zeta, Ne, kT);
+    if (rc || (rc = enqueue_search(ctx, chi, zeta, FERMI_PASSES))) return rc;
+    return enqueue_search(ctx, chi, zeta, 1, true);
 }
 
 int run_fermi(sq_ctx* ctx, const double* chi, const double* zeta, double Ne, double kT, double* mu)
@@ -699,9 +722,8 @@ int run_fermi(sq_ctx* ctx, const double* chi, const double* zeta, double Ne, dou
     int rc = enqueue_search_start(ctx, chi, zeta, Ne, kT);
     if (rc) return rc;
     double st[F_NSTATE];
-    for (int done = 0, n = FERMI_FIRST; done < FERMI_PASSES; done += n) {     // most searches end in the first lot
-        n = std::min(n, FERMI_PASSES - done);
-        if ((rc = enqueue_search(ctx, chi, zeta, n))) return rc;
+    for (int done = 0; done <= FERMI_MAX; done += FERMI_FIRST) {              // most searches end in the first lot
+        if ((rc = enqueue_search(ctx, chi, zeta, FERMI_FIRST))) return rc;
         SQ_CUDA_TRY(cudaMemcpyAsync(st, ctx->d_fermi, sizeof(st), cudaMemcpyDeviceToHost, ctx->stream));
         SQ_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
         if (st[F_DONE] != 0.0) break;
