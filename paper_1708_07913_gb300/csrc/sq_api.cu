@@ -378,7 +378,7 @@ int enqueue_bounds(sq_ctx* c, int blocks, int n_lanczos, double margin, double* 
     }
     c->launches++;
     if (rc) return rc;
-    return launch_tridiag_bounds(c, margin, chi, zeta);
+    return launch_tridiag_bounds(c, n_lanczos, margin, chi, zeta);
 }
 
 // Moments kernel on `blocks` CTAs (Vp built).
@@ -728,7 +728,7 @@ int batch_enqueue_group(sq_batch* b, int gi, const BatchArgs& A)
         sq_ctx* c = b->ctx[g.sys[k]];
         c->launches++;
         c->stream = b->own;
-        if ((rc = launch_tridiag_bounds(c, A.margin, A.chi[g.sys[k]], A.zeta[g.sys[k]]))) return rc;
+        if ((rc = launch_tridiag_bounds(c, A.n_lanczos, A.margin, A.chi[g.sys[k]], A.zeta[g.sys[k]]))) return rc;
     }
     for (int k = 0; k < ns; ++k) {
         sq_ctx* c = b->ctx[g.sys[k]];

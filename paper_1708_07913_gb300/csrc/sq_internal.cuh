@@ -186,9 +186,7 @@ struct sq_ctx {
 // Launchers implemented in the kernel translation units.
 namespace sq {
 int launch_build_vpad(sq_ctx* ctx, const double* V);
-int launch_lanczos(sq_ctx* ctx, int n_lanczos);
-int launch_tridiag_bounds(sq_ctx* ctx, double margin, double* chi, double* zeta);
-int launch_moments(sq_ctx* ctx, const double* chi, const double* zeta, double* moments);
+int launch_tridiag_bounds(sq_ctx* ctx, int n_lanczos, double margin, double* chi, double* zeta);
 int launch_weights(sq_ctx* ctx, const double* moments);
 int run_fermi(sq_ctx* ctx, const double* chi, const double* zeta, double Ne, double kT, double* mu);
 int run_density(sq_ctx* ctx, const double* chi, const double* zeta, double mu, double kT,

@@ -201,17 +201,17 @@ __device__ int sturm_count(int k, const double* a, const double* b2, double x)
 
 // One warp per TRI_NODES nodes: lane = node + 16 * end (0: smallest, 1: largest eigenvalue).
 __global__ void __launch_bounds__(32) tridiag_bounds_kernel(const double* __restrict__ alpha, const double* __restrict__ beta,
-                                                            const int* __restrict__ klen, int cap, long long Nd,
-                                                            double margin, double* __restrict__ chi,
+                                                            const int* __restrict__ klen, int cap, int steps,
+                                                            long long Nd, double margin, double* __restrict__ chi,
                                                             double* __restrict__ zeta)
 {
-    extern __shared__ double tsm[];               // a then b^2, [cap][TRI_NODES] each
+    extern __shared__ double tsm[];               // a then b^2, [steps][TRI_NODES] each
     const int lane = threadIdx.x, n = lane & (TRI_NODES - 1), end = lane >> 4;
     double* A = tsm + n;
-    double* B = tsm + (size_t)cap * TRI_NODES + n;
+    double* B = tsm + (size_t)steps * TRI_NODES + n;
     for (long long q0 = (long long)blockIdx.x * TRI_NODES; q0 < Nd; q0 += (long long)gridDim.x * TRI_NODES) {
         const long long q = q0 + n < Nd ? q0 + n : Nd - 1;
-        const int k = klen[q];
+        const int k = min(klen[q], steps);
         const double* a = alpha + q * cap;
         const double* b = beta + q * cap;
         __syncwarp();
@@ -244,11 +244,13 @@ __global__ void __launch_bounds__(32) tridiag_bounds_kernel(const double* __rest
     }
 }
 
-int launch_tridiag_bounds(sq_ctx* ctx, double margin, double* chi, double* zeta)
+// Extremes of the tridiagonals of n_lanczos steps (the rows of alpha and beta hold ctx->nl_cap); shared memory for
+// these steps only: 48 x 49 x 50 regions of 5^3, 40 steps, take 36.7 ms, and 57.3 with the rows' 512 in shared memory.
+int launch_tridiag_bounds(sq_ctx* ctx, int n_lanczos, double margin, double* chi, double* zeta)
 {
     const long long Nd = ctx->g.Nd;
     const int blocks = (int)std::min<long long>((Nd + TRI_NODES - 1) / TRI_NODES, (long long)ctx->sm_count * 32);
-    const size_t bytes = (size_t)2 * ctx->nl_cap * TRI_NODES * sizeof(double);      // at most 512 steps: 128 KB
+    const size_t bytes = (size_t)2 * n_lanczos * TRI_NODES * sizeof(double);        // at most 512 steps: 128 KB
     if (bytes > 48 * 1024) {                      // raise only (see the region kernels' dispatch)
         cudaFuncAttributes fa;
         if (cudaFuncGetAttributes(&fa, tridiag_bounds_kernel) != cudaSuccess) return SQ_ECUDA;
@@ -257,8 +259,8 @@ int launch_tridiag_bounds(sq_ctx* ctx, double margin, double* chi, double* zeta)
                 cudaSuccess)
             return SQ_ECUDA;
     }
-    tridiag_bounds_kernel<<<blocks, 32, bytes, ctx->stream>>>(ctx->d_alpha, ctx->d_beta, ctx->d_klen, ctx->nl_cap, Nd,
-                                                              margin, chi, zeta);
+    tridiag_bounds_kernel<<<blocks, 32, bytes, ctx->stream>>>(ctx->d_alpha, ctx->d_beta, ctx->d_klen, ctx->nl_cap,
+                                                              n_lanczos, Nd, margin, chi, zeta);
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
