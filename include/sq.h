@@ -299,7 +299,7 @@ int sq_nl_forces_nodes(sq_ctx *ctx, const double *V, const double *chi, const do
  *   system's Fermi level, band energy, entropy energy and electron count
  *   (rho etc. are in the device arrays given to sq_batch_run).  Returns the
  *   first error of any system (SQ_ENOCONV, a latched device error, ...).
- * sq_batch_blocks(b, blocks): HOST array of n: the region-kernel grid chosen
+ * sq_batch_blocks(b, blocks): HOST array of n: the moments kernel's grid chosen
  *   per system (0 = the full persistent grid, and always 0 for the queue
  *   plan); SQ_EINVAL before the first run.
  * sq_batch_destroy(b): releases the batch's streams and graph (NULL: no-op).

@@ -415,7 +415,8 @@ struct sq_batch {
     cudaEvent_t fork = nullptr, ev_in = nullptr, ev_out = nullptr;
     std::vector<cudaEvent_t> join;
     cudaGraphExec_t exec = nullptr;
-    std::vector<int> blocks;                     // region-kernel grid per system (0: the default)
+    // region-kernel grids per system (0: the default): moments, Lanczos (which can run another form)
+    std::vector<int> blocks, blocks_l;
     bool tuned = false;
     // arguments the instantiated graph was captured with
     std::vector<const void*> key_ptr;
@@ -494,17 +495,16 @@ int batch_enqueue_one(sq_batch* b, int i, const BatchArgs& A, int bl, int bm)
 
 // Capture every system's step, each on its own stream forked from and
 // joined back into b->stream, and instantiate the graph.
-int batch_capture_streams(sq_batch* b, const BatchArgs& A, const std::vector<int>& blocks, cudaGraphExec_t* out)
+int batch_capture_streams(sq_batch* b, const BatchArgs& A, const std::vector<int>& blocks,
+                          const std::vector<int>& blocks_l, cudaGraphExec_t* out)
 {
     // grids first: nothing but stream work happens inside the capture
     std::vector<int> bl(b->n), bm(b->n);
     for (int i = 0; i < b->n; ++i) {
         int rc;
         if ((rc = region_blocks(b->ctx[i], 1, &bl[i])) || (rc = region_blocks(b->ctx[i], 0, &bm[i]))) return rc;
-        if (blocks[i] > 0) {
-            bl[i] = std::min(bl[i], blocks[i]);
-            bm[i] = std::min(bm[i], blocks[i]);
-        }
+        if (blocks_l[i] > 0) bl[i] = std::min(bl[i], blocks_l[i]);
+        if (blocks[i] > 0) bm[i] = std::min(bm[i], blocks[i]);
     }
     std::vector<cudaStream_t> saved(b->n);
     for (int i = 0; i < b->n; ++i) saved[i] = b->ctx[i]->stream;
@@ -785,11 +785,11 @@ int batch_capture_queue(sq_batch* b, const BatchArgs& A, cudaGraphExec_t* out)
 }
 
 // Capture launch plan `kind` (SQ_BATCH_STREAMS / _STREAMS_SHARE with the
-// per-system grids `blocks`, or SQ_BATCH_QUEUE with `npi` nodes per item).
-int batch_capture(sq_batch* b, const BatchArgs& A, int kind, const std::vector<int>& blocks, int npi,
-                  cudaGraphExec_t* out)
+// per-system grids `blocks` and `blocks_l`, or SQ_BATCH_QUEUE with `npi` nodes per item).
+int batch_capture(sq_batch* b, const BatchArgs& A, int kind, const std::vector<int>& blocks,
+                  const std::vector<int>& blocks_l, int npi, cudaGraphExec_t* out)
 {
-    if (kind != SQ_BATCH_QUEUE) return batch_capture_streams(b, A, blocks, out);
+    if (kind != SQ_BATCH_QUEUE) return batch_capture_streams(b, A, blocks, blocks_l, out);
     if (b->groups_npi != npi) {
         const int rc = batch_build_queue(b, npi);
         if (rc) return rc;
@@ -815,7 +815,9 @@ int batch_time(sq_batch* b, cudaGraphExec_t g, float* ms)
 
 // Region-kernel grids cut to SM shares proportional to each system's work:
 // nodes x region points x (n_lanczos + n_pl/2) x (1 + the projector share).
-int share_blocks(sq_batch* b, const BatchArgs& A, std::vector<int>* share)
+// The moments and the Lanczos kernel can have different CTAs per SM (the quad
+// form one, the general form several), so each takes the share of its own grid.
+int share_blocks(sq_batch* b, const BatchArgs& A, std::vector<int>* share, std::vector<int>* share_l)
 {
     const int n = b->n;
     std::vector<double> w(n, 0.0);
@@ -826,13 +828,16 @@ int share_blocks(sq_batch* b, const BatchArgs& A, std::vector<int>* share)
         w[i] = (double)c->g.Nd * S * S * S * (A.n_lanczos + c->npl / 2) * (1.0 + proj_pairs(c) * 8.0 / 52.0);
         W += w[i];
     }
-    share->assign(n, 1);
-    for (int i = 0; i < n; ++i) {
-        int bm = 0;
-        int rc = region_blocks(b->ctx[i], 0, &bm);
-        if (rc) return rc;
-        const int per_sm = std::max(1, bm / std::max(1, b->ctx[i]->sm_count));
-        (*share)[i] = std::max(1, (int)std::floor(w[i] / W * b->ctx[i]->sm_count * per_sm));
+    for (int which = 0; which < 2; ++which) {
+        std::vector<int>& s = which == 0 ? *share : *share_l;
+        s.assign(n, 1);
+        for (int i = 0; i < n; ++i) {
+            int blocks = 0;
+            int rc = region_blocks(b->ctx[i], which, &blocks);
+            if (rc) return rc;
+            const int per_sm = std::max(1, blocks / std::max(1, b->ctx[i]->sm_count));
+            s[i] = std::max(1, (int)std::floor(w[i] / W * b->ctx[i]->sm_count * per_sm));
+        }
     }
     return SQ_OK;
 }
@@ -853,8 +858,8 @@ int share_blocks(sq_batch* b, const BatchArgs& A, std::vector<int>* share)
 int batch_tune(sq_batch* b, const BatchArgs& A)
 {
     const int n = b->n;
-    std::vector<int> full(n, 0), share;
-    int rc = share_blocks(b, A, &share);
+    std::vector<int> full(n, 0), share, share_l;
+    int rc = share_blocks(b, A, &share, &share_l);
     if (rc) return rc;
     struct Cand { int kind; int npi; };
     std::vector<Cand> cands;
@@ -872,6 +877,7 @@ int batch_tune(sq_batch* b, const BatchArgs& A)
         b->plan = cands[0].kind;
         b->npi = cands[0].npi;
         b->blocks = b->plan == SQ_BATCH_STREAMS_SHARE ? share : full;
+        b->blocks_l = b->plan == SQ_BATCH_STREAMS_SHARE ? share_l : full;
         b->tuned = true;
         return SQ_OK;
     }
@@ -879,7 +885,8 @@ int batch_tune(sq_batch* b, const BatchArgs& A)
     int pick = 0;
     for (size_t k = 0; k < cands.size(); ++k) {
         cudaGraphExec_t g = nullptr;
-        rc = batch_capture(b, A, cands[k].kind, cands[k].kind == SQ_BATCH_STREAMS_SHARE ? share : full, cands[k].npi, &g);
+        const bool cut = cands[k].kind == SQ_BATCH_STREAMS_SHARE;
+        rc = batch_capture(b, A, cands[k].kind, cut ? share : full, cut ? share_l : full, cands[k].npi, &g);
         float ms = 0.f;
         if (rc == SQ_OK) rc = batch_time(b, g, &ms);
         if (g) cudaGraphExecDestroy(g);
@@ -893,6 +900,7 @@ int batch_tune(sq_batch* b, const BatchArgs& A)
     b->plan = cands[pick].kind;
     b->npi = cands[pick].npi;
     b->blocks = b->plan == SQ_BATCH_STREAMS_SHARE ? share : full;
+    b->blocks_l = b->plan == SQ_BATCH_STREAMS_SHARE ? share_l : full;
     b->tuned = true;
     return SQ_OK;
 }
@@ -1136,6 +1144,7 @@ int sq_batch_create(sq_batch** out, int n, sq_ctx* const* ctxs, void* cuda_strea
     b->st.assign(n, nullptr);
     b->join.assign(n, nullptr);
     b->blocks.assign(n, 0);
+    b->blocks_l.assign(n, 0);
     b->state.assign((size_t)n * FERMI_STATE, 0.0);
     int rc = SQ_OK;
     if (cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -1189,7 +1198,7 @@ int sq_batch_run(sq_batch* b, const double* const* V, double* const* chi, double
         batch_free_graph(b);
         int rc = SQ_OK;
         if (!b->tuned) rc = batch_tune(b, A);
-        if (rc == SQ_OK) rc = batch_capture(b, A, b->plan, b->blocks, b->npi, &b->exec);
+        if (rc == SQ_OK) rc = batch_capture(b, A, b->plan, b->blocks, b->blocks_l, b->npi, &b->exec);
         if (rc) {
             b->exec = nullptr;
             return rc;
