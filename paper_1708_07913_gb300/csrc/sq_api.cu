@@ -346,6 +346,7 @@ int region_blocks(sq_ctx* c, int which, int* blocks)
 int ensure_lanczos_buffers(sq_ctx* c, int n_lanczos)
 {
     if (n_lanczos <= c->nl_cap) return SQ_OK;
+    ++c->moved;
     if (c->d_alpha) cudaFree(c->d_alpha);
     if (c->d_beta) cudaFree(c->d_beta);
     if (c->d_klen) cudaFree(c->d_klen);
@@ -421,6 +422,7 @@ struct sq_batch {
     // arguments the instantiated graph was captured with
     std::vector<const void*> key_ptr;
     std::vector<double> key_val;
+    std::vector<long long> key_moved;            // sq_ctx::moved of every system
     int key_nl = 0;
     double key_margin = -1.0;
     std::vector<double> state;                   // host copy of the Fermi/energy states
@@ -552,6 +554,7 @@ int ensure_scratch(sq_ctx* c, int blocks)
     int rc = dev_alloc(&p, c->scratch_bytes_per_cta * (size_t)blocks);
     if (rc) return rc;
     if (c->d_scratch) cudaFree(c->d_scratch);
+    ++c->moved;
     c->d_scratch = p;
     c->grid_blocks = blocks;
     return SQ_OK;
@@ -1192,8 +1195,14 @@ int sq_batch_run(sq_batch* b, const double* const* V, double* const* chi, double
         cudaGetLastError();
         return SQ_ECUDA;
     }
+    // a graph holds its contexts' buffers: not one that has since been replaced
+    auto moved = [&] {
+        std::vector<long long> v;
+        for (const sq_ctx* c : b->ctx) v.push_back(c->moved);
+        return v;
+    };
     const bool same = b->exec && key == b->key_ptr && kv == b->key_val && n_lanczos == b->key_nl &&
-                      margin == b->key_margin;
+                      margin == b->key_margin && moved() == b->key_moved;
     if (!same) {
         batch_free_graph(b);
         int rc = SQ_OK;
@@ -1206,6 +1215,7 @@ int sq_batch_run(sq_batch* b, const double* const* V, double* const* chi, double
         b->key_ptr = key;
         b->key_val = kv;
         b->key_nl = n_lanczos;
+        b->key_moved = moved();
         b->key_margin = margin;
     }
     if (cudaGraphLaunch(b->exec, b->own) != cudaSuccess || cudaEventRecord(b->ev_out, b->own) != cudaSuccess ||

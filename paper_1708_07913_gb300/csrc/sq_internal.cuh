@@ -181,6 +181,7 @@ struct sq_ctx {
     unsigned* d_count;               // last-block counters
     unsigned* d_err;                 // latched device error bits
     int red_blocks;
+    long long moved;                 // times a buffer that captured work may point to was replaced
 };
 
 // Launchers implemented in the kernel translation units.
