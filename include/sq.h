@@ -503,7 +503,7 @@ enum {
  *   [2] where the per-candidate projector tables live during the general
  *       region kernels: 0 global scratch, 1 all in shared memory, 2 the tables
  *       every step reads in shared memory and the rest in global scratch;
- *   [3] resident CTAs of the general region kernels (per-CTA scratch slices);
+ *   [3] resident CTAs of the general region kernels;
  *   [4] the form that sq_spectral_bounds runs (SQ_FORM_*);
  *   [5] the form that sq_moments runs;
  *   [6] the form that sq_nl_forces runs now (SQ_FORCE_KERNEL is read on every

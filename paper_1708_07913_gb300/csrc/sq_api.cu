@@ -403,6 +403,25 @@ int enqueue_moments(sq_ctx* c, int blocks, const double* chi, const double* zeta
 
 }  // namespace
 
+namespace sq {
+// General per-CTA scratch for at least `blocks` CTAs (a context that runs the
+// quad kernels has none at first, and a queue kernel's grid can be larger than
+// the context's own, e.g. for a system with few nodes).
+// cudaFree synchronises the device, so no kernel still uses the old slices.
+int ensure_scratch(sq_ctx* c, int blocks)
+{
+    if (blocks <= c->grid_blocks) return SQ_OK;
+    void* p = nullptr;
+    int rc = dev_alloc(&p, c->scratch_bytes_per_cta * (size_t)blocks);
+    if (rc) return rc;
+    if (c->d_scratch) cudaFree(c->d_scratch);
+    ++c->moved;
+    c->d_scratch = p;
+    c->grid_blocks = blocks;
+    return SQ_OK;
+}
+}  // namespace sq
+
 // ------------------------------------------------------------------------
 // Batch of independent systems: the whole SCF-iteration step of every
 // context as one CUDA graph, one forked stream per system.
@@ -544,28 +563,12 @@ double proj_pairs(const sq_ctx* c)
     return (c->has_s || c->has_p) ? c->n_atoms * (4.0 / 3.0) * M_PI * c->rnl * c->rnl * c->rnl / cell : 0.0;
 }
 
-// Per-CTA scratch for at least `blocks` CTAs (a queue kernel's grid can be
-// larger than the context's own, e.g. for a system with few nodes).
-// cudaFree synchronises the device, so no kernel still uses the old slices.
-int ensure_scratch(sq_ctx* c, int blocks)
-{
-    if (blocks <= c->grid_blocks) return SQ_OK;
-    void* p = nullptr;
-    int rc = dev_alloc(&p, c->scratch_bytes_per_cta * (size_t)blocks);
-    if (rc) return rc;
-    if (c->d_scratch) cudaFree(c->d_scratch);
-    ++c->moved;
-    c->d_scratch = p;
-    c->grid_blocks = blocks;
-    return SQ_OK;
-}
-
 // The queue plan is open to batches whose contexts all use the single-CTA
 // region kernels (the cluster kernels keep no per-CTA scratch).
 bool queue_available(const sq_batch* b)
 {
     for (const sq_ctx* c : b->ctx)
-        if (c->cl_nc > 0 || !c->d_scratch) return false;
+        if (c->cl_nc > 0) return false;
     return true;
 }
 
@@ -1016,11 +1019,11 @@ int sq_setup_grid(sq_ctx** out, int n1, int n2, int n3, double h, int fd_half_or
         c->nl_extra = 0;
     }
     if ((rcode = region_blocks(c, 0, &bm)) || (rcode = region_blocks(c, 1, &bl))) { free_ctx(c); return rcode; }
-    c->grid_blocks = std::max(bm, bl);
+    c->general_blocks = std::max(bm, bl);
     c->scratch_bytes_per_cta = scratch_layout(m, tsz).total;
-    if (c->cl_nc == 0 &&               // the cluster kernels keep everything in shared memory
-        (rcode = dev_alloc(&c->d_scratch, c->scratch_bytes_per_cta * c->grid_blocks))) { free_ctx(c); return rcode; }
     if ((rcode = select_quad_kernels(c))) { free_ctx(c); return rcode; }
+    if (c->cl_nc == 0 &&               // the cluster kernels keep everything in shared memory
+        (rcode = ensure_scratch(c, std::max(c->quad[0] ? 0 : bm, c->quad[1] ? 0 : bl)))) { free_ctx(c); return rcode; }
     c->red_blocks = c->sm_count * 4;
     if ((rcode = dev_alloc(&c->d_W, sizeof(double) * c->g.Nd * (npl + 1))) ||
         (rcode = dev_alloc(&c->d_red, sizeof(double) * RED_VALUES * c->red_blocks)) ||
@@ -1118,7 +1121,7 @@ int sq_context_info(const sq_ctx* c, int* info, int n)
     info[0] = c->g.m;
     info[1] = c->ccap;
     info[2] = c->nl_mode;
-    info[3] = c->grid_blocks;
+    info[3] = std::max(c->general_blocks, c->grid_blocks);
     for (int i = 4; i < n && i < 6; ++i)
         info[i] = c->cl_nc > 0 ? SQ_FORM_CLUSTER : c->quad[i == 4 ? 1 : 0] ? SQ_FORM_QUAD : SQ_FORM_GENERAL;
     if (n > 6) info[6] = force_form(c);

@@ -209,7 +209,7 @@ RegionForceLayout region_force_layout(int S, int n_atoms, size_t tsz)
 // Grid of the region form (0: not available for this context).
 int region_force_blocks(const sq_ctx* c, long long nq, size_t* extra)
 {
-    if (c->cl_nc > 0 || !c->d_scratch) return 0;        // the cluster kernels keep no per-CTA scratch
+    if (c->cl_nc > 0) return 0;                         // the cluster kernels keep no per-CTA scratch
     const char* env = getenv("SQ_FORCE_KERNEL");
     if (env && strcmp(env, "legacy") == 0) return 0;
     *extra = force_coef_bytes(c->npl) + c->nl_extra;
@@ -218,7 +218,7 @@ int region_force_blocks(const sq_ctx* c, long long nq, size_t* extra)
     const int rc = c->precision == SQ_FP32 ? force_region_config_f32(c->g.m, *extra, &bps, &smem)
                                            : force_region_config_f64(c->g.m, *extra, &bps, &smem);
     if (rc || bps < 1) return 0;
-    long long b = std::min<long long>((long long)bps * c->sm_count, c->grid_blocks);
+    long long b = std::min<long long>((long long)bps * c->sm_count, std::max(c->general_blocks, c->grid_blocks));
     return (int)std::min<long long>(b, nq);
 }
 
@@ -403,7 +403,7 @@ int nl_forces(sq_ctx* c, const double* V, const double* chi, const double* zeta,
         rc = launch_force_quad(c, L, ws->buf, qblocks, extra, chi, zeta, mu, kT, nodes, nq, forces);
     } else if (rblocks > 0) {
         const RegionForceLayout L = region_force_layout(S, c->n_atoms, tsz);
-        if ((rc = force_workspace(c, L.total * (size_t)rblocks, &ws))) return rc;
+        if ((rc = ensure_scratch(c, rblocks)) || (rc = force_workspace(c, L.total * (size_t)rblocks, &ws))) return rc;
         if ((rc = launch_build_vpad(c, V))) return rc;
         rc = c->precision == SQ_FP32
                  ? launch_force_region<float>(c, L, ws->buf, rblocks, extra, chi, zeta, mu, kT, nodes, nq, forces)

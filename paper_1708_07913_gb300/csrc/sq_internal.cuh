@@ -165,8 +165,10 @@ struct sq_ctx {
     void* d_qscratch;
     uint32_t* d_qmask;               // support rows as column masks (QuadArgs::mask)
     size_t q_stride;
-    // per-CTA scratch
-    int grid_blocks;                 // resident CTAs used for the region kernels
+    // per-CTA scratch of the general kernels, for those that the context runs
+    // (ensure_scratch: more when a queue or the region force form needs it)
+    int general_blocks;              // their resident CTAs
+    int grid_blocks;                 // slices allocated
     size_t scratch_bytes_per_cta;
     void* d_scratch;
     // Lanczos tridiagonals
@@ -201,6 +203,7 @@ constexpr int FERMI_STATE = 12;      // doubles of the device Fermi/energy state
 int fermi_result(const double* st_host, double* mu, double* eb, double* es, double* ne);
 int launch_proj_tables(sq_ctx* ctx, const double* d_R);
 int launch_support_masks(sq_ctx* ctx, int* most_row_entries);
+int ensure_scratch(sq_ctx* ctx, int blocks);
 int force_form(const sq_ctx* ctx);       // SQ_FORM_* that nl_forces runs
 }  // namespace sq
 

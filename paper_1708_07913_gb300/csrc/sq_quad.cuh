@@ -99,7 +99,7 @@ __host__ __device__ inline QuadScratch quad_scratch(int m, int ccap, int lb)
     L.ent = o;   o = align256(o + (size_t)ccap * quad_recs(lb) * 16);
     L.yt = o;    o = align256(o + (m == QD_MMAX ? (size_t)ccap * quad_nyp(lb) * 16 : 0));
     L.ab = o;    o = align256(o + (m == QD_MMAX ? (size_t)(ccap * (lb + 1) + 1) * 16 : 0));
-    L.total = o;
+    L.total = ccap > 0 ? o : L.list;     // without projectors only the potential
     return L;
 }
 
