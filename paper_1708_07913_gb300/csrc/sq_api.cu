@@ -274,9 +274,10 @@ int cluster_launch(sq_ctx* c, int which, const RegionArgs<float>& a, int blocks)
 }
 
 // FP32 quad kernels (sq_quad.cuh) for this context: every region half-width
-// that has one, unless its projector tables do not fit next to the vector or
-// SQ_REGION_KERNEL=cta in the environment asks for the general kernels.
-// Allocates their per-CTA scratch and sets c->quad.
+// that has one, unless its projector tables do not fit next to the vector,
+// their per-CTA scratch cannot be allocated (it can be twice the general
+// kernels') or SQ_REGION_KERNEL=cta in the environment asks for the general
+// kernels.  Allocates that scratch and sets c->quad.
 int select_quad_kernels(sq_ctx* c)
 {
     c->quad[0] = c->quad[1] = 0;
@@ -290,15 +291,14 @@ int select_quad_kernels(sq_ctx* c)
         if (rc == SQ_EUNSUPPORTED) return SQ_OK;
         if (rc) return rc;
     }
-    int rc;
     if (has_nl) {
-        int most = 0;
-        if ((rc = dev_alloc(&c->d_qmask, sizeof(uint32_t) * (c->lb * c->lb * (size_t)c->n_atoms + 1)))) return rc;
+        int rc, most = 0;
+        if (dev_alloc(&c->d_qmask, sizeof(uint32_t) * (c->lb * c->lb * (size_t)c->n_atoms + 1))) return SQ_OK;
         if ((rc = launch_support_masks(c, &most))) return rc;
         if (most > ENTRIES_PER_ROW) return SQ_OK;          // the general kernels refuse such rows
     }
     c->q_stride = quad_scratch(c->g.m, has_nl ? c->ccap : 0, has_nl ? c->lb : 0).total;
-    if ((rc = dev_alloc(&c->d_qscratch, c->q_stride * (size_t)c->sm_count))) return rc;   // one CTA per SM, a queue's too
+    if (dev_alloc(&c->d_qscratch, c->q_stride * (size_t)c->sm_count)) return SQ_OK;       // one CTA per SM, a queue's too
     c->quad[0] = 1;
     c->quad[1] = !has_nl || c->g.m >= QD_MIN_NL_LANCZOS;
     return SQ_OK;

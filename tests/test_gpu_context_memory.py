@@ -1,5 +1,6 @@
 """Device memory of a context: the quad kernels' per-CTA scratch in place of the
-general kernels', not on top of it."""
+general kernels', not on top of it, and the general kernels when it cannot be had."""
+import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -72,3 +73,41 @@ def test_region_force_form_gets_its_scratch_on_first_use(monkeypatch):
     sq.sq_destroy(ctx)
     scale = float(F["region"].abs().max())
     assert scale > 1e-6 and float((F[""] - F["region"]).abs().max()) <= 2 * FP32_FORCE * scale
+
+
+def test_general_kernels_when_the_quad_scratch_cannot_be_had(monkeypatch):
+    import torch
+    from paper_1708_07913_gb300 import sq
+    m, atoms = 14, 1
+    shape, h = GRIDS[m % 2], 0.5
+    _, V, _ = _inputs(shape, h, 1, 40 + m)
+    nq = V.size
+    V = torch.from_numpy(V).cuda()
+    chi = torch.full((nq,), 20.0, dtype=torch.float64, device="cuda")
+    zeta = torch.full_like(chi, 60.0)
+    bounds = [torch.empty_like(chi), torch.empty_like(chi)]
+    mom = {}
+    took = {}
+    for kernel in ("", "cta", "", "cta"):                # the first ones also load the kernels
+        ctx, took[kernel] = _setup(monkeypatch, kernel, m, atoms)
+        mom[kernel] = torch.empty(nq, 17, dtype=torch.float64, device="cuda")
+        sq.sq_spectral_bounds(ctx, V, *bounds, 8, 0.02)
+        sq.sq_moments(ctx, V, chi, zeta, mom[kernel])
+        sq.sq_sync(ctx)
+        sq.sq_destroy(ctx)
+    assert took[""] > took["cta"] + 80 * MB
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    ballast = torch.empty(torch.cuda.mem_get_info()[0] - took["cta"] - 40 * MB, dtype=torch.uint8, device="cuda")
+    try:
+        ctx, _ = _setup(monkeypatch, "", m, atoms)
+        info = sq.sq_context_info(ctx)
+        assert info["moments"] == info["lanczos"] == sq.FORM_GENERAL
+        sq.sq_moments(ctx, V, chi, zeta, mom[""])
+        sq.sq_sync(ctx)
+        sq.sq_destroy(ctx)
+    finally:
+        del ballast
+        torch.cuda.empty_cache()
+    assert float((mom[""] - mom["cta"]).abs().max()) < 2e-5       # FP32, as in test_gpu_parity.py
+    assert np.isfinite(mom[""].cpu().numpy()).all()
