@@ -286,7 +286,8 @@ int select_quad_kernels(sq_ctx* c)
     if (env && strcmp(env, "cta") == 0) return SQ_OK;
     const bool has_nl = c->n_atoms > 0;
     if (c->g.m < (has_nl ? QD_MIN_NL : QD_MIN_LOCAL)) return SQ_OK;
-    for (int which = 0; which < 2; ++which) {
+    const bool lanczos = !has_nl || c->g.m >= QD_MIN_NL_LANCZOS;
+    for (int which = 0; which < (lanczos ? 2 : 1); ++which) {
         const int rc = quad_config(c->g.m, which, has_nl, c->ccap, c->lb, c->npl, &c->q_smem[which]);
         if (rc == SQ_EUNSUPPORTED) return SQ_OK;
         if (rc) return rc;
@@ -300,7 +301,7 @@ int select_quad_kernels(sq_ctx* c)
     c->q_stride = quad_scratch(c->g.m, has_nl ? c->ccap : 0, has_nl ? c->lb : 0).total;
     if (dev_alloc(&c->d_qscratch, c->q_stride * (size_t)c->sm_count)) return SQ_OK;       // one CTA per SM, a queue's too
     c->quad[0] = 1;
-    c->quad[1] = !has_nl || c->g.m >= QD_MIN_NL_LANCZOS;
+    c->quad[1] = lanczos;
     return SQ_OK;
 }
 

@@ -92,20 +92,6 @@ struct CnnGrid {
     long long N;
 };
 
-// node index of p + d on the periodic grid
-__device__ inline long long cnn_nb(const CnnGrid& g, int i, int j, int k, int dx, int dy, int dz)
-{
-    return (long long)cnn_wrap(i + dx, g.n1) +
-           (long long)g.n1 * ((long long)cnn_wrap(j + dy, g.n2) + (long long)g.n2 * cnn_wrap(k + dz, g.n3));
-}
-
-__device__ inline void cnn_ijk(const CnnGrid& g, long long p, int& i, int& j, int& k)
-{
-    i = (int)(p % g.n1);
-    j = (int)((p / g.n1) % g.n2);
-    k = (int)(p / ((long long)g.n1 * g.n2));
-}
-
 // x0 = (V - shift) / scale, stored in T
 template <typename T>
 __global__ void cnn_input_kernel(CnnGrid g, const double* __restrict__ V, double shift, double scale, T* __restrict__ x0)

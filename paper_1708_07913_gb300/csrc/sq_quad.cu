@@ -7,7 +7,10 @@ template <int M>
 static int config_m(int which, bool has_nl, int ccap, int lb, int npl, size_t* smem)
 {
     const size_t bytes = quad_smem_bytes<M>(has_nl, ccap, lb, which == 0 ? npl : 0);
-    const void* fn = which == 0 ? (const void*)quad_kernel<M, false> : (const void*)quad_kernel<M, true>;
+    const void* fn = nullptr;
+    if (which == 0) fn = (const void*)quad_kernel<M, false>;
+    else if constexpr (quad_has_lanczos(M)) fn = (const void*)quad_kernel<M, true>;
+    if (!fn) return SQ_EUNSUPPORTED;
     cudaFuncAttributes fa;                       // the limit only ever grows (see sq_region_dispatch.cuh)
     if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) {
         cudaGetLastError();
@@ -27,7 +30,8 @@ template <int M>
 static int launch_m(int which, const QuadArgs& a, size_t smem, int blocks, cudaStream_t st)
 {
     if (which == 0) quad_kernel<M, false><<<blocks, QD_NT, smem, st>>>(a);
-    else quad_kernel<M, true><<<blocks, QD_NT, smem, st>>>(a);
+    else if constexpr (quad_has_lanczos(M)) quad_kernel<M, true><<<blocks, QD_NT, smem, st>>>(a);
+    else return SQ_EUNSUPPORTED;
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
 

@@ -51,6 +51,7 @@ constexpr int QD_MMAX = 15;                  // region half-widths 7 .. 15 have 
 // 29^3; 5e-6 at most without projectors).  Those keep the general kernel's
 // rounding, whose own run-to-run spread is ten times smaller.
 constexpr int QD_MIN_NL = 7, QD_MIN_LOCAL = 8, QD_MIN_NL_LANCZOS = 11;
+constexpr bool quad_has_lanczos(int m) { return m >= QD_MIN_LOCAL || m >= QD_MIN_NL_LANCZOS; }
 constexpr int QD_NT = 512, QD_NW = 16;
 constexpr int QD_KMAX = 4 * ENTRIES_PER_ROW;  // list length per (quad, row pair, plane pair): four full rows
 constexpr int QD_ZERO = 504;                  // 8 TMEM columns of zeros: the planes beyond the region

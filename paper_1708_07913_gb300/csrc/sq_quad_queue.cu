@@ -8,14 +8,18 @@ template <int M>
 static int launch_m(int which, const QuadQueueArgs& q, size_t smem, int blocks, cudaStream_t st)
 {
     if (which == 0) quad_queue_kernel<M, false><<<blocks, QD_NT, smem, st>>>(q);
-    else quad_queue_kernel<M, true><<<blocks, QD_NT, smem, st>>>(q);
+    else if constexpr (quad_has_lanczos(M)) quad_queue_kernel<M, true><<<blocks, QD_NT, smem, st>>>(q);
+    else return SQ_EUNSUPPORTED;
     return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ECUDA;
 }
 
 template <int M>
 static int config_m(int which, size_t smem)
 {
-    const void* fn = which == 0 ? (const void*)quad_queue_kernel<M, false> : (const void*)quad_queue_kernel<M, true>;
+    const void* fn = nullptr;
+    if (which == 0) fn = (const void*)quad_queue_kernel<M, false>;
+    else if constexpr (quad_has_lanczos(M)) fn = (const void*)quad_queue_kernel<M, true>;
+    if (!fn) return SQ_EUNSUPPORTED;
     cudaFuncAttributes fa;                       // the limit only ever grows (see sq_region_dispatch.cuh)
     if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) {
         cudaGetLastError();
