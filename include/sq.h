@@ -208,16 +208,27 @@ int sq_density_energy_noalloc(int n1, int n2, int n3, double h, int npl,
  *              overwritten; may be NULL when the context has no projectors
  * The recurrence vectors, D and the projector inner products are in the
  * context's precision (FP32 or FP64); the coefficients c^j and the final
- * contraction are FP64.  The recurrence runs on the machinery of the region
- * kernels (one CTA per node, vectors in shared memory); in FP32 its
- * projector update adds with shared-memory atomics, so repeated calls agree
- * to FP32 rounding, and FP64 results repeat bit for bit.  Where that form
- * does not fit the context (or with SQ_FORCE_KERNEL=legacy in the
- * environment) a first form with every vector in global scratch runs, which
- * repeats bit for bit in both precisions.  Allocates, on first use, about
- * (resident CTAs) x (s (2m+1)^3 + 12 KB + 24 n_atoms) bytes of workspace in
- * the context (s = 4 or 8 bytes; the first form: 2 x SMs x (4 s (2m+1)^3 +
- * (384 + 128 s) (2m+1)^2 + (24 + 4 s) ccap + 24 n_atoms)).
+ * contraction are FP64.  Three forms (sq_context_info reports which runs):
+ *   SQ_FORM_QUAD     FP32 contexts whose moments run the quad kernels, unless
+ *                    the coefficients of a large npl do not fit beside the
+ *                    tables: the quad kernels' recurrence, fixed order
+ *                    everywhere, so repeated calls agree bit for bit;
+ *   SQ_FORM_GENERAL  else, or with SQ_FORCE_KERNEL=region in the environment:
+ *                    the machinery of the general region kernels (one CTA per
+ *                    node, vectors in shared memory); in FP32 its projector
+ *                    update adds with shared-memory atomics, so repeated calls
+ *                    agree to FP32 rounding, and FP64 results repeat bit for
+ *                    bit;
+ *   SQ_FORM_FIRST    where that does not fit the context, or with
+ *                    SQ_FORCE_KERNEL=legacy: every vector in global scratch,
+ *                    repeats bit for bit in both precisions.
+ * Allocates, on first use, workspace in the context, about
+ *   quad     SMs x (4096 (2m+1) + 12 KB + 24 n_atoms) + 8 (npl+1)^2 bytes;
+ *   general  (resident CTAs) x (s (2m+1)^3 + 12 KB + 24 n_atoms) bytes (s = 4 or
+ *            8), and the general kernels' per-CTA scratch where the context
+ *            has none yet;
+ *   first    2 x SMs x (4 s (2m+1)^3 + (384 + 128 s) (2m+1)^2 + (24 + 4 s) ccap +
+ *            24 n_atoms) bytes.
  * Synchronises the stream; a projector-table overflow (more candidates or
  * row entries than the tables hold) returns SQ_ECAPACITY. */
 int sq_nl_forces(sq_ctx *ctx, const double *V, const double *chi, const double *zeta,
@@ -240,7 +251,7 @@ int sq_nl_forces_nodes(sq_ctx *ctx, const double *V, const double *chi, const do
  * bounds, moments, Fermi level and density/energies, as the single-system
  * calls above define them -- for every context in it as ONE CUDA graph
  * launch, so that systems of uneven size, region and temperature share the
- * GPU and the launch-bound Fermi-level bisections of the systems overlap.
+ * GPU and the launch-bound Fermi-level searches of the systems overlap.
  * The contexts of a batch must be distinct.
  *
  * sq_batch_create(out, n, ctxs, cuda_stream)

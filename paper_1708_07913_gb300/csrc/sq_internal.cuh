@@ -179,7 +179,7 @@ struct sq_ctx {
     // quadrature weights and reductions
     double* d_W;                     // [npl+1][Nd]
     double* d_red;                   // block partials
-    double* d_fermi;                 // bisection state
+    double* d_fermi;                 // state of the Fermi search
     unsigned* d_count;               // last-block counters
     unsigned* d_err;                 // latched device error bits
     int red_blocks;

@@ -4,7 +4,7 @@
 //     region of influence, Section 3.1)
 //   * extreme eigenvalues of the Lanczos tridiagonals (Section 3.2)
 //   * quadrature weights by discrete orthogonality (Eq. cqj)
-//   * Fermi level by bisection on the electron count (Section 3.2)
+//   * Fermi level by a bracketing search on the electron count (Section 3.2)
 //   * density, band energy and entropy (Eqs. ElectronDensity, Eband, Entropy)
 // Every global sum is deterministic: per-block tree sums in a fixed order,
 // then the last block to finish adds the block partials in index order.

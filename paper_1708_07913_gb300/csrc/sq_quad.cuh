@@ -48,8 +48,13 @@ constexpr int QD_MMAX = 15;                  // region half-widths 7 .. 15 have 
 // FP32 steps leave unconverged move with the rounding, and the moments with them
 // (largest change over the moments' rms between the two kernels, seven seeded
 // systems each: 1e-2 at 17^3, 2e-3 at 19^3, 5e-4 at 21^3, 8e-5 at 23^3, 2e-5 at
-// 29^3; 5e-6 at most without projectors).  Those keep the general kernel's
-// rounding, whose own run-to-run spread is ten times smaller.
+// 29^3; 5e-6 at most without projectors).  Those stay on the general kernel, whose
+// own run-to-run spread is ten times smaller, so that results there stay what they
+// were.  It is no more exact: rms error of zeta against FP64 Lanczos over the rms
+// of zeta, seven seeded systems each, general / quad: 1.94e-5 / 1.93e-5 at 15^3,
+// 1.02e-5 / 0.98e-5 at 17^3, 8.6e-6 / 8.8e-6 at 19^3, 6.4e-6 / 6.4e-6 at 21^3,
+// 3.6e-6 / 3.6e-6 at 23^3; largest error 3.5e-3 / 3.6e-3 at 15^3, 7.8e-5 / 6.9e-5 at
+// 23^3.
 constexpr int QD_MIN_NL = 7, QD_MIN_LOCAL = 8, QD_MIN_NL_LANCZOS = 11;
 constexpr bool quad_has_lanczos(int m) { return m >= QD_MIN_LOCAL || m >= QD_MIN_NL_LANCZOS; }
 constexpr int QD_NT = 512, QD_NW = 16;

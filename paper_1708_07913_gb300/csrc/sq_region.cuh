@@ -75,8 +75,11 @@ struct Geo {
 // The second vector of the recurrence (t^{i-1}, later t^{i+1}) or of Lanczos
 // (v_old, then w): in shared memory with the same padded layout as the first
 // when two vectors fit (DB = true), otherwise unpadded in per-CTA global
-// scratch.  Only the thread that owns a column (or a row, in the projector
-// pre-pass) touches it, so its layout needs no halo.
+// scratch.  Every pass touches a point of it in one thread only, so its layout
+// needs no halo; but that thread is the point's row's in the projector update,
+// its column's in the sweep and, in FP64, where the sweep packs the columns
+// (Owner), another one in the vector passes of Lanczos: a barrier stands between
+// any two of these passes.
 template <int M, bool DB>
 struct Sec {
     using G = Geo<M>;
