@@ -135,6 +135,15 @@ KERNEL_SOURCES = ("sq_internal.cuh", "sq_region.cuh", "sq_region_dispatch.cuh", 
                   "sq_region_f64.cu", "sq_quad.cuh", "sq_quad.cu")
 
 
+def region_kernel_name(solver, step):
+    """The kernel that runs `step` ("lanczos" or "moments") of a context."""
+    from paper_1708_07913_gb300 import sq
+    info = sq.sq_context_info(solver.ctx)
+    if info[step] == sq.FORM_QUAD:
+        return f"quad_kernel<{info['m']}, {'true' if step == 'lanczos' else 'false'}>"
+    return f"{'cl_' if info[step] == sq.FORM_CLUSTER else ''}{step}_kernel"
+
+
 def source_sha():
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1708_07913_gb300", "csrc")
@@ -426,7 +435,8 @@ def run_gb300(a):
         peak = sms * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
     else:
         peak = 1.25 * sms / SM_COUNT_GB300 * sm_max / 2070.0     # FP64 at GB300's published 1.25 TFLOP/s
-    kern = {"lanczos_kernel": (flops_lanczos(wl), t_bounds), "moments_kernel": (flops_moments(wl), t_mom)}
+    kern = {region_kernel_name(solver, "lanczos"): (flops_lanczos(wl), t_bounds),
+            region_kernel_name(solver, "moments"): (flops_moments(wl), t_mom)}
     dom = max(kern, key=lambda k: kern[k][1])
     achieved = kern[dom][0] / kern[dom][1] / 1e12
     traffic = None
@@ -684,7 +694,7 @@ def run_force(a):
     spectral bounds and Fermi level of one SQ step computed first (not
     timed).  One step = one force evaluation."""
     import torch
-    from paper_1708_07913_gb300 import SQ_FP32, SQ_FP64, SQSolver, build
+    from paper_1708_07913_gb300 import SQ_FP32, SQ_FP64, SQSolver, build, sq
 
     name = a.workload[len("force_"):]
     dev = torch.device("cuda:0")
@@ -735,7 +745,7 @@ def run_force(a):
     t = float(np.mean(times))
     nt = touched_nodes(wl, s.positions)
     S = 2 * wl.m + 1
-    quad = prec == SQ_FP32 and 7 <= wl.m <= 15 and not os.environ.get("SQ_FORCE_KERNEL")    # the form that runs by default
+    form = sq.sq_context_info(solver.ctx)["forces"]
     units = nt * wl.npl
     flops = nt * wl.npl * S ** 3 * (FORCE_FLOPS_PER_POINT + NL_FLOPS_PER_PAIR * nl_pairs_per_point(wl))
     peaks = json.load(open(PEAKS_PATH)) if os.path.exists(PEAKS_PATH) else {}
@@ -757,17 +767,17 @@ def run_force(a):
                                f"a projector support",
                    "precision": ("FP32 recurrence, D and projector sums; FP64 coefficients and contraction"
                                  if prec == SQ_FP32 else "FP64 throughout"),
-                   "kernel": ("first form, current vector in shared memory (SQ_FORCE_KERNEL=legacy, SQ_FORCE_SMEM=1)"
-                              if os.environ.get("SQ_FORCE_KERNEL") == "legacy" and os.environ.get("SQ_FORCE_SMEM") == "1"
-                              else "first form, vectors in global scratch (SQ_FORCE_KERNEL=legacy)"
-                              if os.environ.get("SQ_FORCE_KERNEL") == "legacy"
-                              else "quad form (the quad kernels' recurrence with D in global scratch)" if quad
+                   "kernel": ("first form, current vector in shared memory (SQ_FORCE_SMEM=1)"
+                              if form == sq.FORM_FIRST and os.environ.get("SQ_FORCE_SMEM") == "1"
+                              else "first form, vectors in global scratch" if form == sq.FORM_FIRST
+                              else "quad form (the quad kernels' recurrence with D in global scratch)"
+                              if form == sq.FORM_QUAD
                               else "region form (the region kernels' recurrence with D in global scratch)"),
                    "l2": "flushed between timed steps (256 MB write)",
                    "parallelism": "single GPU"},
         "forces_max_abs": float(F.abs().max().item()),
-        "roofline": {"kernel": ("nl_force_kernel" if os.environ.get("SQ_FORCE_KERNEL") == "legacy"
-                                else "quad_force_kernel" if quad else "force_region_kernel"),
+        "roofline": {"kernel": ("nl_force_kernel" if form == sq.FORM_FIRST
+                                else "quad_force_kernel" if form == sq.FORM_QUAD else "force_region_kernel"),
                      "bound": "alu", "achieved": flops / t / 1e12, "peak": peak,
                      "unit": "TFLOP/s", "frac": flops / t / 1e12 / peak, "traffic": None, "peak_basis": basis},
         "e2e": {"value": units / float(np.median(e2e)), "unit": FORCE_UNIT,
